@@ -1,9 +1,10 @@
 // Ising model with the spin-flip policy (Sec. II) on periodic square and simple cubic
 // lattices, multi-spin coded: one 32-bit word holds 32 consecutive sites of one colour of
-// one row (x direction) of one replica. A thread takes one word position for a group of four
-// replicas (the four words of one Philox block per site): it builds, bit-sliced, the count
-// of neighbours aligned with each spin, draws one Philox block per site, and decides 128
-// flips against integer thresholds. Magnetization and bond sums are popcounts.
+// one row (x direction) of one replica. A thread takes one word position (or, on small
+// lattices, a part of it) for a group of four replicas, the four words of one Philox block per
+// site: it compares every word with the acceptance thresholds of the step, which fills one
+// bit mask per threshold, builds the count of neighbours aligned with each spin bit-sliced,
+// and combines both into the flips of the 32 sites. Magnetization and bond sums are popcounts.
 //
 // Threshold: accept iff dE <= 0 or w < ceil(exp(-beta dE) 2^32), which for an integer w is
 // exactly w 2^-32 < exp(-beta dE). The host computes exp in FP64 with the same expression
@@ -29,26 +30,29 @@ constexpr uint32_t kPurposeIsingInit = 0x90000u;
 constexpr int kIsingThreads = 256;
 constexpr int kMaxIsingReplicas = 512;
 
-struct IsingThr {          // one replica at one temperature/field step
-    uint32_t thr[14];      // class s * (z + 1) + a: accept iff w < thr (when not always)
-    uint32_t always;       // bit per class: dE <= 0
-    uint32_t pad;
-};
-
-struct IsingRun {
-    uint32_t t, rec, mcs, pad;
-    const IsingThr *thr;          // [n_steps][R]
-    const double *h;              // [n_steps][R]
-    double *hist;                 // [records][R][2]
-    unsigned long long *acc;      // [R][2]: up spins, aligned bonds (colour-1 ends)
+// One threshold of one replica at one temperature/field step, with the spins it decides: those
+// whose count of aligned neighbours has the bits selected by (x0, x1, x2) and whose own bit is
+// selected by x3 (any when `any` is all ones). A class (own spin, aligned neighbours) whose flip is
+// always accepted has no entry. Every field but neg is 0 or all ones.
+struct __align__(16) IsingThr {
+    uint32_t neg;         // 2^32 - thr: w + neg carries iff w >= thr (the flip is rejected)
+    uint32_t x0, x1, x2;  // match = (p0 ^ x0) & (p1 ^ x1) & (p2 ^ x2) & (((own ^ x3) & on) | any)
+    uint32_t x3, on, any;
+    uint32_t never;       // thr = 0: rejected whatever w
 };
 
 struct IsingPassArgs {
     uint32_t *spins;
-    IsingRun *run;
-    uint64_t seed;
-    int64_t rows;        // L^(dims-1)
-    int32_t L, KW, R, c, inst_base;
+    const IsingThr *thr;      // [R][NQ] of this step
+    unsigned long long *acc;  // [R][2]: up spins, aligned bonds (colour-1 ends) of the current MCS
+    uint32_t *ticket;         // blocks done in the colour-1 pass (zero between passes)
+    const double *h;          // [R] fields of this step
+    double *hist;             // [R][2] record of this MCS
+    double J;
+    int64_t n;                // sites
+    uint32_t rk0[10], rk1[10];  // Philox round keys (seed + r * Weyl constants)
+    uint32_t t, rows, L, KW;  // MCS counter; rows = L^(dims-1), KW = L / 64 words per row and colour
+    int32_t R, c, inst_base;
 };
 
 __host__ __device__ inline int64_t word_index(int r, int c, int64_t row, int kw, int64_t rows, int KW) {
@@ -64,122 +68,144 @@ __device__ __forceinline__ void slice_add(uint32_t x, uint32_t &p0, uint32_t &p1
     p2 ^= c1;
 }
 
-template <int DIMS>
-__global__ void __launch_bounds__(kIsingThreads) ising_pass_kernel(const IsingPassArgs a) {
-    constexpr int Z = 2 * DIMS;
-    __shared__ IsingThr s_thr[kMaxIsingReplicas];
-    IsingRun *rs = a.run;
-    const uint32_t t = rs->t;
-    const uint32_t step = rs->rec / rs->mcs;
-    for (int i = threadIdx.x; i < a.R; i += blockDim.x) s_thr[i] = rs->thr[(int64_t)step * a.R + i];
-    __syncthreads();
-    const int L = a.L, KW = a.KW, c = a.c, oc = 1 - c;
-    const int64_t rows = a.rows, per_g = rows * KW, n_items = (int64_t)(a.R / 4) * per_g;
-    const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
-    const int lane = threadIdx.x & 31;
-    uint32_t *S = a.spins;
-    unsigned long long up[4] = {0, 0, 0, 0}, al[4] = {0, 0, 0, 0};
-    int g_cur = -1;
-    auto flush = [&]() {  // warp-uniform: all lanes share g_cur
-        for (int j = 0; j < 4; ++j) {
-            unsigned long long u = up[j], v = al[j];
-            for (int off = 16; off > 0; off >>= 1) {
-                u += __shfl_xor_sync(0xFFFFFFFFu, u, off);
-                v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-            }
-            if (lane == 0 && g_cur >= 0) {
-                atomicAdd(&rs->acc[(g_cur * 4 + j) * 2], u);
-                atomicAdd(&rs->acc[(g_cur * 4 + j) * 2 + 1], v);
-            }
-            up[j] = 0;
-            al[j] = 0;
-        }
-    };
-    // n_items and the stride are multiples of 32, and so is per_g: a warp's items share g
-    for (int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; item < n_items;
-         item += (int64_t)gridDim.x * blockDim.x) {
-        const int g = (int)(item / per_g);
-        if (g != g_cur) {
-            flush();
-            g_cur = g;
-        }
-        const int64_t rem = item - (int64_t)g * per_g;
-        const int64_t row = rem / KW;
-        const int kw = (int)(rem - row * KW);
-        const int y = (int)(row % L), zc = DIMS == 3 ? (int)(row / L) : 0;
-        const int off = (y + zc + c) & 1;
-        const int64_t rym = (int64_t)((y + L - 1) % L) + (int64_t)L * zc, ryp = (int64_t)((y + 1) % L) + (int64_t)L * zc;
-        const int64_t rzm = DIMS == 3 ? (int64_t)y + (int64_t)L * ((zc + L - 1) % L) : 0;
-        const int64_t rzp = DIMS == 3 ? (int64_t)y + (int64_t)L * ((zc + 1) % L) : 0;
-        const int kws = off == 0 ? (kw + KW - 1) % KW : (kw + 1) % KW;
-        uint32_t own[4], nb[4][Z], p0[4], p1[4], p2[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = g * 4 + j;
-            own[j] = S[word_index(r, c, row, kw, rows, KW)];
-            const uint32_t xa = S[word_index(r, oc, row, kw, rows, KW)];
-            const uint32_t xb = S[word_index(r, oc, row, kws, rows, KW)];
-            nb[j][0] = xa;                                                      // x neighbour at the same k
-            nb[j][1] = off == 0 ? (xa << 1) | (xb >> 31) : (xa >> 1) | (xb << 31);  // k - 1 or k + 1
-            nb[j][2] = S[word_index(r, oc, rym, kw, rows, KW)];
-            nb[j][3] = S[word_index(r, oc, ryp, kw, rows, KW)];
-            if (DIMS == 3) {
-                nb[j][4] = S[word_index(r, oc, rzm, kw, rows, KW)];
-                nb[j][5] = S[word_index(r, oc, rzp, kw, rows, KW)];
-            }
-            p0[j] = p1[j] = p2[j] = 0u;
-#pragma unroll
-            for (int q = 0; q < Z; ++q) slice_add(~(own[j] ^ nb[j][q]), p0[j], p1[j], p2[j]);
-        }
-        uint32_t flip[4] = {0u, 0u, 0u, 0u};
-        const uint32_t group = (uint32_t)(a.inst_base >> 2) + (uint32_t)g;
-        const int64_t site0 = (int64_t)L * row + off + (int64_t)kw * 64;  // x = 2 (32 kw + b) + off
-        for (int b = 0; b < 32; ++b) {
-            const uint32_t site = (uint32_t)(site0 + 2 * b);
-            const uint4 w = philox10(make_uint4(site, t, group, kPurposeIsing), k0, k1);
-            const uint32_t wj[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int cls = (int)((own[j] >> b) & 1u) * (Z + 1) + (int)((p0[j] >> b) & 1u) +
-                                2 * (int)((p1[j] >> b) & 1u) + 4 * (int)((p2[j] >> b) & 1u);
-                const IsingThr &T = s_thr[g * 4 + j];
-                const bool acc = ((T.always >> cls) & 1u) || wj[j] < T.thr[cls];
-                flip[j] |= (uint32_t)acc << b;
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t nw = own[j] ^ flip[j];
-            if (flip[j]) S[word_index(g * 4 + j, c, row, kw, rows, KW)] = nw;
-            up[j] += (unsigned long long)__popc(nw);
-            if (c == 1) {  // each bond counted at its colour-1 end, after the update
-#pragma unroll
-                for (int q = 0; q < Z; ++q) al[j] += (unsigned long long)__popc(~(nw ^ nb[j][q]));
-            }
-        }
-    }
-    flush();
+// R = 2R + carry(w + neg): appends the decision bit "w >= thr" to a mask in two instructions.
+__device__ __forceinline__ void append_reject(uint32_t &mask, uint32_t w, uint32_t neg) {
+    asm("{\n\t.reg .u32 s;\n\tadd.cc.u32 s, %1, %2;\n\taddc.u32 %0, %0, %0;\n\t}" : "+r"(mask) : "r"(w), "r"(neg));
 }
 
-// After both passes: (E, M) of every replica into the history; the counters are cleared and
-// the MCS counter and record index advance. One block, one thread per replica.
-__global__ void ising_reduce_kernel(IsingRun *rs, int32_t R, int64_t n, int32_t Z, double J) {
-    const uint32_t rec = rs->rec, step = rec / rs->mcs;
-    for (int r = threadIdx.x; r < R; r += blockDim.x) {
-        const unsigned long long upc = rs->acc[r * 2], alc = rs->acc[r * 2 + 1];
-        const int64_t M = 2 * (int64_t)upc - n;
-        const int64_t bsum = 2 * (int64_t)alc - (int64_t)Z * (n / 2);
-        const double h = rs->h[(int64_t)step * R + r];
-        double *o = rs->hist + ((int64_t)rec * R + r) * 2;
-        o[0] = __dsub_rn(__dmul_rn(-J, (double)bsum), __dmul_rn(h, (double)M));
-        o[1] = (double)M;
-        rs->acc[r * 2] = 0;
-        rs->acc[r * 2 + 1] = 0;
+// One colour pass. Bound by integer issue (Philox: 18 wide multiplies and 20 logic operations
+// per site for four replicas; the spins are a bit each, so memory moves little). Every bit of the
+// decision is therefore kept bit-sliced: two instructions per attempt and threshold (NQ = Z/2
+// thresholds without a field, at most Z + 1 with one) in place of extracting the site's class
+// and looking its threshold up. The random part needs no spin: it runs before
+// griddepcontrol.wait, so it overlaps the tail of the pass before (programmatic dependent
+// launch). S threads share a word position (32 / S sites each) on lattices too small to fill the
+// GPU. 960^2 x 32 replicas: 90 us per MCS with class look-ups and a reduction kernel of its own
+// (42 instructions per attempt), @@NOW@@ now.
+template <int DIMS, int NQ, int S>
+__global__ void __launch_bounds__(kIsingThreads) ising_pass_kernel(const IsingPassArgs a) {
+    constexpr int Z = 2 * DIMS, NB = 32 / S;
+    __shared__ uint32_t s_sum[8];
+    __shared__ bool s_last;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (threadIdx.x < 8) s_sum[threadIdx.x] = 0u;
+    const uint32_t g = blockIdx.y, L = a.L, KW = a.KW, rows = a.rows, plane = rows * KW;
+    const uint32_t idx = blockIdx.x * kIsingThreads + threadIdx.x;  // below 2^25 * 8 + 256
+    const uint32_t item = idx / S, sub = idx % S;
+    const bool active = item < plane;  // whole warps (plane is a multiple of 64)
+    const int c = a.c, oc = 1 - c;
+    uint32_t up[4] = {0u, 0u, 0u, 0u}, al[4] = {0u, 0u, 0u, 0u};
+    __syncthreads();
+    if (active) {
+        const uint32_t row = item / KW, kw = item - row * KW;
+        const uint32_t zc = DIMS == 3 ? row / L : 0u, y = row - zc * L;
+        const uint32_t off = (y + zc + (uint32_t)c) & 1u;
+        const IsingThr *T = a.thr + (size_t)g * 4 * NQ;
+        uint32_t rej[4][NQ], neg[4][NQ];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                rej[j][q] = 0u;
+                neg[j][q] = __ldg(&T[j * NQ + q].neg);
+            }
+        const uint32_t group = (uint32_t)(a.inst_base >> 2) + g;
+        const uint32_t site0 = L * row + off + kw * 64u + 2u * NB * sub;  // x = 2 (32 kw + b) + off
+#pragma unroll 2
+        for (int b = NB - 1; b >= 0; --b) {  // the last appended bit is bit 0
+            uint4 w = make_uint4(site0 + 2u * (uint32_t)b, a.t, group, kPurposeIsing);
+#pragma unroll
+            for (int r = 0; r < 10; ++r) {
+                const uint32_t lo0 = 0xD2511F53u * w.x, hi0 = __umulhi(0xD2511F53u, w.x);
+                const uint32_t lo1 = 0xCD9E8D57u * w.z, hi1 = __umulhi(0xCD9E8D57u, w.z);
+                w = make_uint4(hi1 ^ w.y ^ a.rk0[r], lo1, hi0 ^ w.w ^ a.rk1[r], lo0);
+            }
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                append_reject(rej[0][q], w.x, neg[0][q]);
+                append_reject(rej[1][q], w.y, neg[1][q]);
+                append_reject(rej[2][q], w.z, neg[2][q]);
+                append_reject(rej[3][q], w.w, neg[3][q]);
+            }
+        }
+        // every spin of the pass before is final from here on; read through L2, since a block of
+        // that pass may have left older words in this SM's L1
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const uint32_t rym = y == 0u ? row + L - 1u : row - 1u, ryp = y + 1u == L ? row + 1u - L : row + 1u;
+        const uint32_t rzm = zc == 0u ? row + L * (L - 1u) : row - L, rzp = zc + 1u == L ? row - L * (L - 1u) : row + L;
+        const uint32_t kws = off == 0u ? (kw == 0u ? KW - 1u : kw - 1u) : (kw + 1u == KW ? 0u : kw + 1u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint32_t *So = a.spins + word_index((int)(g * 4) + j, c, 0, 0, rows, (int)KW);
+            const uint32_t *Sn = a.spins + word_index((int)(g * 4) + j, oc, 0, 0, rows, (int)KW);
+            const uint32_t own = __ldcg(So + item);
+            const uint32_t xa = __ldcg(Sn + item), xb = __ldcg(Sn + row * KW + kws);
+            uint32_t nb[Z];
+            nb[0] = xa;                                                        // x neighbour at the same k
+            nb[1] = off == 0u ? (xa << 1) | (xb >> 31) : (xa >> 1) | (xb << 31);  // k - 1 or k + 1
+            nb[2] = __ldcg(Sn + rym * KW + kw);
+            nb[3] = __ldcg(Sn + ryp * KW + kw);
+            if (DIMS == 3) {
+                nb[Z - 2] = __ldcg(Sn + rzm * KW + kw);
+                nb[Z - 1] = __ldcg(Sn + rzp * KW + kw);
+            }
+            uint32_t p0 = 0u, p1 = 0u, p2 = 0u;
+#pragma unroll
+            for (int q = 0; q < Z; ++q) slice_add(~(own ^ nb[q]), p0, p1, p2);
+            uint32_t reject = 0u;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const uint4 ta = __ldg((const uint4 *)&T[j * NQ + q]), tb = __ldg((const uint4 *)&T[j * NQ + q] + 1);
+                const uint32_t match =
+                    (p0 ^ ta.y) & (p1 ^ ta.z) & (p2 ^ ta.w) & (((own ^ tb.x) & tb.y) | tb.z);
+                reject |= match & ((S > 1 ? rej[j][q] << (NB * sub) : rej[j][q]) | tb.w);
+            }
+#pragma unroll
+            for (int o = 1; o < S; o <<= 1) reject |= __shfl_xor_sync(0xFFFFFFFFu, reject, o);
+            const uint32_t flip = ~reject, nw = own ^ flip;
+            if (S == 1 || sub == 0u) {
+                if (flip) So[item] = nw;
+                up[j] = (uint32_t)__popc(nw);
+                // bonds aligned after the update, counted at their colour-1 ends: a aligned
+                // neighbours stay a, or become Z - a under a flip
+                if (c == 1)
+                    al[j] = (uint32_t)(__popc(p0) + 2 * __popc(p1) + 4 * __popc(p2) + Z * __popc(flip) -
+                                       2 * (__popc(p0 & flip) + 2 * __popc(p1 & flip) + 4 * __popc(p2 & flip)));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t u = __reduce_add_sync(0xFFFFFFFFu, up[j]);
+            if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum[2 * j], u);
+            if (c == 1) {
+                const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, al[j]);
+                if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum[2 * j + 1], v);
+            }
+        }
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // the counters below are the pass before's too
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        rs->t = rs->t + 1;
-        rs->rec = rec + 1;
+    if (threadIdx.x < 8 && s_sum[threadIdx.x])
+        atomicAdd(&a.acc[(size_t)(g * 4 + threadIdx.x / 2) * 2 + (threadIdx.x & 1)], (unsigned long long)s_sum[threadIdx.x]);
+    if (c == 0) return;
+    // the colour-1 pass ends the MCS: its last block writes every replica's record (E, M) and
+    // clears the counters (no other block touches them before this grid has ended)
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(a.ticket, 1u) == gridDim.x * gridDim.y - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *a.ticket = 0u;
+    for (int r = (int)threadIdx.x; r < a.R; r += kIsingThreads) {
+        const unsigned long long upc = __ldcg(&a.acc[r * 2]), alc = __ldcg(&a.acc[r * 2 + 1]);
+        const int64_t M = 2 * (int64_t)upc - a.n;
+        const int64_t bsum = 2 * (int64_t)alc - (int64_t)Z * (a.n / 2);
+        a.hist[r * 2] = __dsub_rn(__dmul_rn(-a.J, (double)bsum), __dmul_rn(a.h[r], (double)M));
+        a.hist[r * 2 + 1] = (double)M;
+        a.acc[r * 2] = 0ull;
+        a.acc[r * 2 + 1] = 0ull;
     }
 }
 
@@ -226,12 +252,12 @@ struct vegas_ising {
     int64_t n = 0, rows = 0;
     int32_t KW = 0, Z = 0;
     uint32_t *d_spins = nullptr;
-    IsingRun *d_run = nullptr;
     IsingThr *d_thr = nullptr;
+    uint32_t *d_ticket = nullptr;
     double *d_h = nullptr, *d_hist = nullptr;
     unsigned long long *d_acc = nullptr;
     size_t thr_cap = 0, hist_cap = 0;
-    int grid = 1;
+    int split = 1;  // threads per word position
     std::vector<std::vector<double>> hist;  // per replica: records * 2
     int64_t records = 0;
     uint32_t t = 0;
@@ -270,7 +296,7 @@ vegas_status ising_host_exception(vegas_ising *c) {
     } while (0)
 
 void ising_free(vegas_ising *c) {
-    void *bufs[] = {c->d_spins, c->d_run, c->d_thr, c->d_h, c->d_hist, c->d_acc};
+    void *bufs[] = {c->d_spins, c->d_thr, c->d_ticket, c->d_h, c->d_hist, c->d_acc};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -282,13 +308,75 @@ vegas_status ising_usable(vegas_ising *c) {
     return VEGAS_OK;
 }
 
-void launch_ising_pass(vegas_ising *c, int colour, cudaStream_t st) {
-    IsingPassArgs a{c->d_spins, c->d_run, c->opt.seed, c->rows, c->opt.L, c->KW, c->opt.replicas, colour,
-                    c->opt.inst_base};
-    if (c->opt.dims == 3)
-        ising_pass_kernel<3><<<c->grid, kIsingThreads, 0, st>>>(a);
-    else
-        ising_pass_kernel<2><<<c->grid, kIsingThreads, 0, st>>>(a);
+using IsingFn = void (*)(IsingPassArgs);
+
+template <int DIMS, int NQ>
+IsingFn select_split(int split) {
+    if (split == 1) return ising_pass_kernel<DIMS, NQ, 1>;
+    return split == 2 ? ising_pass_kernel<DIMS, NQ, 2> : split == 4 ? ising_pass_kernel<DIMS, NQ, 4> : ising_pass_kernel<DIMS, NQ, 8>;
+}
+
+// nq: thresholds per replica, Z / 2 or Z + 1.
+cudaError_t launch_ising_pass(const vegas_ising *c, IsingPassArgs &a, int nq, int colour) {
+    a.c = colour;
+    const IsingFn f = c->opt.dims == 3 ? (nq == 3 ? select_split<3, 3>(c->split) : select_split<3, 7>(c->split))
+                                       : (nq == 2 ? select_split<2, 2>(c->split) : select_split<2, 5>(c->split));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((c->rows * c->KW * c->split + kIsingThreads - 1) / kIsingThreads), (unsigned)(a.R / 4));
+    cfg.blockDim = dim3(kIsingThreads);
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, a);
+}
+
+// The thresholds of one replica at one step, into t[Z + 1]; returns how many there are. At most
+// Z + 1: of the four classes with a or Z - a aligned neighbours (a < Z / 2), dE > 0 holds for at
+// most two, and of the two with Z / 2 for at most one. Without a field the two spin directions
+// share a threshold, which leaves Z / 2.
+int ising_thresholds(double J, double beta, double hh, int Z, IsingThr *t) {
+    uint32_t thr[2][8];
+    bool always[2][8];
+    for (int sb = 0; sb < 2; ++sb)
+        for (int al = 0; al <= Z; ++al) {
+            const double si = sb ? 1.0 : -1.0;
+            const double sum = sb ? (double)(2 * al - Z) : (double)(Z - 2 * al);
+            const double dE = 2.0 * si * (J * sum + hh);
+            always[sb][al] = true;
+            thr[sb][al] = 0u;
+            if (dE <= 0.0) continue;
+            // accept iff w < x = exp(-beta dE) 2^32 (w integer): iff w < ceil(x)
+            const double x = std::ceil(std::exp(-(beta * dE)) * 4294967296.0);
+            if (x >= 4294967296.0) continue;
+            always[sb][al] = false;
+            thr[sb][al] = (uint32_t)x;
+        }
+    int nq = 0;
+    auto add = [&](int al, uint32_t x, uint32_t own1, uint32_t any) {
+        IsingThr e{};
+        e.neg = 0u - x;
+        e.x0 = (al & 1) ? 0u : ~0u;
+        e.x1 = (al & 2) ? 0u : ~0u;
+        e.x2 = (al & 4) ? 0u : ~0u;
+        e.x3 = own1 ? 0u : ~0u;
+        e.on = ~0u;
+        e.any = any;
+        e.never = x == 0u ? ~0u : 0u;
+        if (nq < Z + 1) t[nq] = e;
+        ++nq;
+    };
+    for (int al = 0; al <= Z; ++al) {
+        if (!always[0][al] && !always[1][al] && thr[0][al] == thr[1][al]) {
+            add(al, thr[0][al], 0u, ~0u);
+        } else {
+            if (!always[0][al]) add(al, thr[0][al], 0u, 0u);
+            if (!always[1][al]) add(al, thr[1][al], 1u, 0u);
+        }
+    }
+    return nq;
 }
 
 }  // namespace
@@ -365,16 +453,15 @@ static vegas_status ising_create(const vegas_ising_options *opt, vegas_ising **o
              }
              const size_t words = (size_t)o.replicas * 2 * (size_t)c->rows * (size_t)c->KW;
              ICK(c, cudaMalloc(&c->d_spins, words * sizeof(uint32_t)));
-             ICK(c, cudaMalloc(&c->d_run, sizeof(IsingRun)));
+             ICK(c, cudaMalloc(&c->d_ticket, sizeof(uint32_t)));
              ICK(c, cudaMalloc(&c->d_acc, sizeof(unsigned long long) * 2 * o.replicas));
-             c->device_bytes = (int64_t)(words * 4 + sizeof(IsingRun) + 16 * (size_t)o.replicas);
+             c->device_bytes = (int64_t)(words * 4 + sizeof(uint32_t) + 16 * (size_t)o.replicas);
              ICK(c, cudaMemsetAsync(c->d_acc, 0, sizeof(unsigned long long) * 2 * o.replicas, c->stream));
-             int nb = 0;
-             ICK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                        &nb, o.dims == 3 ? ising_pass_kernel<3> : ising_pass_kernel<2>, kIsingThreads, 0));
+             ICK(c, cudaMemsetAsync(c->d_ticket, 0, sizeof(uint32_t), c->stream));
              const int64_t items = (int64_t)(o.replicas / 4) * c->rows * c->KW;
-             c->grid = (int)std::max<int64_t>(1, std::min<int64_t>((items + kIsingThreads - 1) / kIsingThreads,
-                                                                   (int64_t)c->sm_count * std::max(nb, 1)));
+             // a thread per word position once they give every SM 16 warps; below, up to 8 threads
+             // share one (a warp alone needs about 7 us for the 32 Philox blocks of a word)
+             while (c->split < 8 && items * c->split < (int64_t)c->sm_count * 512) c->split *= 2;
              const int64_t init_items = 2 * items;
              const int ig = (int)std::min<int64_t>((init_items + 255) / 256, (int64_t)c->sm_count * 8);
              ising_init_kernel<<<ig, 256, 0, c->stream>>>(c->d_spins, o.seed, c->rows, o.L, c->KW, o.replicas, o.dims,
@@ -416,35 +503,25 @@ extern "C" vegas_status vegas_ising_run(vegas_ising *c, const double *T, const d
         if ((int64_t)c->t + (int64_t)n_steps * mcs >= (int64_t)UINT32_MAX)
             return ifail(c, VEGAS_EINVAL, "global MCS counter would exceed 32 bits");
         const int R = c->opt.replicas, Z = c->Z;
-        std::vector<IsingThr> thr((size_t)n_steps * R);
+        // thresholds [step][R][Z + 1], compacted below to each step's count
+        std::vector<IsingThr> thr((size_t)n_steps * R * (Z + 1));
+        std::vector<int> nq((size_t)n_steps, Z / 2);
         std::vector<double> hv((size_t)n_steps * R);
         for (int r = 0; r < R; ++r)
             for (int s = 0; s < n_steps; ++s) {
                 const double Tv = T[(int64_t)r * n_steps + s], hh = h[(int64_t)r * n_steps + s];
                 if (!(Tv > 0.0) || !std::isfinite(Tv)) return ifail(c, VEGAS_EINVAL, "T must be finite and > 0");
                 if (!std::isfinite(hh)) return ifail(c, VEGAS_EINVAL, "h must be finite");
-                const double beta = 1.0 / Tv;
-                IsingThr &e = thr[(size_t)s * R + r];
-                std::memset(&e, 0, sizeof e);
-                for (int sb = 0; sb < 2; ++sb)
-                    for (int al = 0; al <= Z; ++al) {
-                        const double si = sb ? 1.0 : -1.0;
-                        const double sum = sb ? (double)(2 * al - Z) : (double)(Z - 2 * al);
-                        const double dE = 2.0 * si * (c->opt.J * sum + hh);
-                        const int cls = sb * (Z + 1) + al;
-                        if (dE <= 0.0) {
-                            e.always |= 1u << cls;
-                            continue;
-                        }
-                        // accept iff w < x = exp(-beta dE) 2^32 (w integer): iff w < ceil(x)
-                        const double x = std::ceil(std::exp(-(beta * dE)) * 4294967296.0);
-                        if (x >= 4294967296.0)
-                            e.always |= 1u << cls;
-                        else
-                            e.thr[cls] = (uint32_t)x;
-                    }
+                const int k = ising_thresholds(c->opt.J, 1.0 / Tv, hh, Z, &thr[((size_t)s * R + r) * (Z + 1)]);
+                if (k > Z + 1) return ifail(c, VEGAS_EINVAL, "more acceptance thresholds than classes with dE > 0");
+                if (k > Z / 2) nq[(size_t)s] = Z + 1;
                 hv[(size_t)s * R + r] = hh;
             }
+        for (int s = 0; s < n_steps; ++s)
+            if (nq[(size_t)s] == Z / 2)
+                for (int r = 0; r < R; ++r)
+                    for (int q = 0; q < Z / 2; ++q)
+                        thr[(size_t)s * R * (Z + 1) + (size_t)r * (Z / 2) + q] = thr[((size_t)s * R + r) * (Z + 1) + q];
         ICK(c, cudaSetDevice(c->device));
         const int64_t nrec = (int64_t)n_steps * mcs;
         if (thr.size() > c->thr_cap) {
@@ -454,7 +531,7 @@ extern "C" vegas_status vegas_ising_run(vegas_ising *c, const double *T, const d
             c->d_h = nullptr;
             c->thr_cap = 0;
             ICK(c, cudaMalloc(&c->d_thr, sizeof(IsingThr) * thr.size()));
-            ICK(c, cudaMalloc(&c->d_h, sizeof(double) * thr.size()));
+            ICK(c, cudaMalloc(&c->d_h, sizeof(double) * hv.size()));
             c->thr_cap = thr.size();
         }
         const size_t hneed = (size_t)nrec * R * 2;
@@ -467,8 +544,21 @@ extern "C" vegas_status vegas_ising_run(vegas_ising *c, const double *T, const d
         }
         ICK(c, cudaMemcpyAsync(c->d_thr, thr.data(), sizeof(IsingThr) * thr.size(), cudaMemcpyHostToDevice, c->stream));
         ICK(c, cudaMemcpyAsync(c->d_h, hv.data(), sizeof(double) * hv.size(), cudaMemcpyHostToDevice, c->stream));
-        IsingRun rs{c->t, 0u, (uint32_t)mcs, 0u, c->d_thr, c->d_h, c->d_hist, c->d_acc};
-        ICK(c, cudaMemcpyAsync(c->d_run, &rs, sizeof rs, cudaMemcpyHostToDevice, c->stream));
+        IsingPassArgs pa{};
+        pa.spins = c->d_spins;
+        pa.acc = c->d_acc;
+        pa.ticket = c->d_ticket;
+        pa.J = c->opt.J;
+        pa.n = c->n;
+        pa.rows = (uint32_t)c->rows;
+        pa.L = (uint32_t)c->opt.L;
+        pa.KW = (uint32_t)c->KW;
+        pa.R = R;
+        pa.inst_base = c->opt.inst_base;
+        for (uint32_t q = 0; q < 10; ++q) {
+            pa.rk0[q] = (uint32_t)c->opt.seed + q * 0x9E3779B9u;
+            pa.rk1[q] = (uint32_t)(c->opt.seed >> 32) + q * 0xBB67AE85u;
+        }
         std::vector<cudaEvent_t> ev;
         if (c->opt.timing) {
             ev.resize((size_t)nrec * 4);
@@ -478,14 +568,17 @@ extern "C" vegas_status vegas_ising_run(vegas_ising *c, const double *T, const d
         ICK(c, cudaEventCreate(&e0));
         ICK(c, cudaEventCreate(&e1));
         ICK(c, cudaEventRecord(e0, c->stream));
-        const int rthreads = std::min(std::max(32, (R + 31) / 32 * 32), 512);
         for (int64_t m = 0; m < nrec; ++m) {
+            const int64_t s = m / mcs;
+            pa.thr = c->d_thr + (size_t)s * R * (Z + 1);
+            pa.h = c->d_h + s * R;
+            pa.hist = c->d_hist + m * R * 2;
+            pa.t = c->t + (uint32_t)m;
             for (int colour = 0; colour < 2; ++colour) {
                 if (c->opt.timing) ICK(c, cudaEventRecord(ev[(size_t)m * 4 + 2 * colour], c->stream));
-                launch_ising_pass(c, colour, c->stream);
+                ICK(c, launch_ising_pass(c, pa, nq[(size_t)s], colour));
                 if (c->opt.timing) ICK(c, cudaEventRecord(ev[(size_t)m * 4 + 2 * colour + 1], c->stream));
             }
-            ising_reduce_kernel<<<1, rthreads, 0, c->stream>>>(c->d_run, R, c->n, Z, c->opt.J);
         }
         ICK(c, cudaGetLastError());
         ICK(c, cudaEventRecord(e1, c->stream));
@@ -503,7 +596,7 @@ extern "C" vegas_status vegas_ising_run(vegas_ising *c, const double *T, const d
         for (auto &x : ev) cudaEventDestroy(x);
         c->last_run_ms = ms;
         c->sweep_ms += sw;
-        c->kernel_launches += nrec * 3;
+        c->kernel_launches += nrec * 2;
         c->sweep_launches += nrec * 2;
         std::vector<double> hh(hneed);
         ICK(c, cudaMemcpy(hh.data(), c->d_hist, sizeof(double) * hneed, cudaMemcpyDeviceToHost));
