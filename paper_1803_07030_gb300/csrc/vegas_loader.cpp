@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <thread>
 #include <unordered_map>
 
 #include "vegas_internal.h"
@@ -163,27 +164,58 @@ bool load_sample(const vegas_sample &s, LoadedSample &L, std::string &err, bool 
             if (s.col[e] == i) { *Jout = s.J[e]; return 1; }
         return 0;
     };
-    for (int32_t i = 0; i < n; ++i) {
-        const int64_t b = s.row_ptr[i], d = s.row_ptr[i + 1] - b;
-        if (d > kScan) {
-            const auto &v = sorted.at(i);
-            for (size_t q = 0; q < v.size(); ++q) {
-                if (v[q].first == i) { err = at("self-link at site", i); return false; }
-                if (q > 0 && v[q].first == v[q - 1].first) { err = at("duplicate link at site", i); return false; }
+    // rows [i0, i1); the first fault found goes to e1
+    auto check_rows = [&](int32_t i0, int32_t i1, std::string &e1) -> bool {
+        for (int32_t i = i0; i < i1; ++i) {
+            const int64_t b = s.row_ptr[i], d = s.row_ptr[i + 1] - b;
+            if (d > kScan) {
+                const auto &v = sorted.at(i);
+                for (size_t q = 0; q < v.size(); ++q) {
+                    if (v[q].first == i) { e1 = at("self-link at site", i); return false; }
+                    if (q > 0 && v[q].first == v[q - 1].first) { e1 = at("duplicate link at site", i); return false; }
+                }
+            } else {
+                for (int64_t e = b; e < b + d; ++e) {
+                    if (s.col[e] == i) { e1 = at("self-link at site", i); return false; }
+                    for (int64_t f = b; f < e; ++f)
+                        if (s.col[f] == s.col[e]) { e1 = at("duplicate link at site", i); return false; }
+                }
             }
-        } else {
             for (int64_t e = b; e < b + d; ++e) {
-                if (s.col[e] == i) { err = at("self-link at site", i); return false; }
-                for (int64_t f = b; f < e; ++f)
-                    if (s.col[f] == s.col[e]) { err = at("duplicate link at site", i); return false; }
+                double Jr = 0.0;
+                if (!find_in_row(s.col[e], i, &Jr)) { e1 = at("link without its reverse, edge", e); return false; }
+                if (Jr != s.J[e]) { e1 = at("J not symmetric, edge", e); return false; }
             }
         }
-        for (int64_t e = b; e < b + d; ++e) {
-            double Jr = 0.0;
-            if (!find_in_row(s.col[e], i, &Jr)) { err = at("link without its reverse, edge", e); return false; }
-            if (Jr != s.J[e]) { err = at("J not symmetric, edge", e); return false; }
+        return true;
+    };
+    // a random read per link and, on long rows, a search: on several host threads for large samples,
+    // reporting the fault of the lowest site as one thread does
+    const int nt = (int)std::min<int64_t>({16, (int64_t)std::max(1u, std::thread::hardware_concurrency()), E / 65536 + 1});
+    std::vector<std::string> faults((size_t)nt);
+    std::vector<char> ok((size_t)nt, 0);
+    auto part = [&](int k) {
+        try {
+            ok[(size_t)k] = check_rows((int32_t)((int64_t)n * k / nt), (int32_t)((int64_t)n * (k + 1) / nt), faults[(size_t)k]);
+        } catch (...) {  // no memory for the message
         }
+    };
+    {
+        std::vector<std::thread> th;
+        int k = 1;
+        try {
+            for (; k < nt; ++k) th.emplace_back(part, k);
+        } catch (...) {
+        }
+        part(0);
+        for (; k < nt; ++k) part(k);  // threads that could not be started
+        for (std::thread &t : th) t.join();
     }
+    for (int k = 0; k < nt; ++k)
+        if (!ok[(size_t)k]) {
+            err = faults[(size_t)k].empty() ? "checking the links failed" : faults[(size_t)k];
+            return false;
+        }
     sorted.clear();
 
     // parameters (defaults: s = 1, n = +z, k = 0, e = +z, kc = 0)
