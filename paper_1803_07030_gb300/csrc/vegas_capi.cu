@@ -10,9 +10,11 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "vegas_internal.h"
+#include "vegas_tile.h"
 
 using namespace vegas;
 
@@ -120,11 +122,20 @@ struct vegas_ctx {
     int cluster_cs = 0, cluster_n = 0, cluster_threads = 256;
     // cooperative sweep
     bool coop_eligible = false;
+    int32_t max_class_sites = 0;  // one sample: its widest colour class
     CoopArgs coop{};
     int coop_grid = 1;
     int coop_grid_max = 1;  // every block the GPU holds at once, capped by the widest class and max_blocks
     GridBarrier *d_bar = nullptr;
     double *d_coop_partial = nullptr;
+    // tiled form of the cooperative sweep (FP32 rows of at most kEllRow links, parts that fit in
+    // shared memory); the grid-barrier form serves the others
+    bool tile_ok = false;
+    bool use_tile = false;  // the cooperative sweep runs it (not while the autotuner times the sweeps)
+    TileArgs tile{};
+    int tile_threads = 0;
+    size_t tile_smem_bytes = 0;
+    std::vector<void *> tile_bufs;
     // wavefront sweep: both classes of an MCS in one launch
     WaveArgs wave{};
     int wave_grid = 1;
@@ -216,6 +227,7 @@ void free_all(vegas_ctx *c) {
                     c->d_fold_deps, c->d_fold_deg, c->d_fold_cnt};
     for (void *b : bufs)
         if (b) cudaFree(b);
+    for (void *b : c->tile_bufs) cudaFree(b);
     for (LaunchGroup &lg : c->launches) {
         if (lg.d_args) cudaFree(lg.d_args);
         if (lg.d_first) cudaFree(lg.d_first);
@@ -347,8 +359,23 @@ void enqueue_resident(vegas_ctx *c, cudaStream_t st, int32_t n) {
     launch_advance(c->d_run, n, st);
 }
 
-// One cooperative launch for n MCS of the current step; the run state advances afterwards.
+// Kernels that the cooperative sweep launches for n MCS of a step.
+int64_t coop_kernels(const vegas_ctx *c, int32_t n) {
+    return c->use_tile ? 3 * (int64_t)((n + kTileMcs - 1) / kTileMcs) : 2;
+}
+
+// One cooperative launch for n MCS of the current step (the tiled form: one per kTileMcs MCS, and
+// one that writes their records); the run state advances afterwards.
 void enqueue_coop(vegas_ctx *c, cudaStream_t st, int32_t n) {
+    if (c->use_tile) {
+        TileArgs a = c->tile;
+        for (int32_t m = 0; m < n; m += kTileMcs) {
+            a.mcs = std::min(kTileMcs, n - m);
+            if (launch_tile(a, c->tile_threads, c->tile_smem_bytes, st) != 0) return;
+            launch_advance(c->d_run, a.mcs, st);
+        }
+        return;
+    }
     cudaMemsetAsync(c->d_bar, 0, sizeof(GridBarrier), st);
     CoopArgs a = c->coop;
     a.mcs = n;
@@ -543,6 +570,77 @@ bool class1_block_deps(const SampleInfo &si, const LoadedSample &l, int bs, int 
         last[(size_t)q] = nd > 0 ? dq[nd - 1] : 0;
     }
     return true;
+}
+
+// The tiled form of the cooperative sweep for the context's one FP32 sample: parts of at least
+// kTilePerClass sites of the widest class, at most one block per SM over all replicas. Leaves
+// tile_ok unset when its rows are longer than kEllRow or a part does not fit in shared memory.
+vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
+    const SampleInfo &si = c->samples[0];
+    const vegas_options &o = c->opt;
+    int64_t max_deg = 0;
+    for (int32_t g = 0; g < si.n; ++g) max_deg = std::max(max_deg, l.row_ptr[(size_t)g + 1] - l.row_ptr[(size_t)g]);
+    int32_t widest = 1;
+    for (int32_t q = 0; q < si.n_colours; ++q) widest = std::max(widest, si.cstart[(size_t)q + 1] - si.cstart[(size_t)q]);
+    c->max_class_sites = widest;
+    const int blocks = o.max_blocks > 0 ? std::min(c->sm_count, o.max_blocks) : c->sm_count;
+    TileShape ts{};
+    ts.n = si.n;
+    ts.n_colours = si.n_colours;
+    ts.parts = std::min(blocks / c->R, (widest + kTilePerClass - 1) / kTilePerClass);
+    ts.width = si.uniform_degree == 6 ? 6 : kEllRow;
+    ts.site_off = si.site_off;
+    ts.cstart = l.cstart.data();
+    ts.lower_mode = l.lower_mode.data();
+    ts.col = l.col.data();
+    ts.orig = l.orig.data();
+    ts.row_ptr = l.row_ptr.data();
+    ts.J = l.J.data();
+    TilePlan plan;
+    // a part's spins take 12 bytes per site (a quick bound before the plan is made)
+    if (max_deg > kEllRow || ts.parts < 1 || 12 * (int64_t)(si.n / ts.parts) > kResSmemBytes || !tile_plan(ts, plan))
+        return VEGAS_OK;
+    TileArgs &a = c->tile;
+    a = TileArgs{};
+    a.pass = c->passes[0].args;
+    a.P = ts.parts;
+    a.n_colours = si.n_colours;
+    a.n_mail = plan.n_mail;
+    a.width = ts.width;
+    a.cubic = std::any_of(l.k_cub.begin(), l.k_cub.end(), [](double x) { return x != 0.0; });
+    a.timeout_ns = o.timeout_ns > 0 ? o.timeout_ns : 2000000000LL;
+    a.skip_block = o.fault_inject == 1 ? 0 : -1;
+    for (uint32_t q = 0; q < 10; ++q) {
+        a.rk0[q] = (uint32_t)o.seed + q * 0x9E3779B9u;
+        a.rk1[q] = (uint32_t)(o.seed >> 32) + q * 0xBB67AE85u;
+    }
+    c->tile_threads = tile_shape(a, ts, plan, &c->tile_smem_bytes);
+    cudaGetLastError();
+    if (c->tile_threads == 0) return VEGAS_OK;
+    auto up = [&](auto *&p, const void *src, size_t bytes) {
+        void *d = nullptr;
+        const cudaError_t e = dalloc(c, &d, std::max<size_t>(bytes, 16));
+        if (e != cudaSuccess) return e;
+        c->tile_bufs.push_back(d);
+        p = (std::remove_reference_t<decltype(p)>)d;
+        return src && bytes > 0 ? cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, c->stream) : cudaSuccess;
+    };
+    const size_t words = (size_t)kTileMcs * c->R * ts.parts;
+    CK(c, up(a.parts, plan.parts.data(), plan.parts.size() * sizeof(TilePart)));
+    CK(c, up(a.classes, plan.classes.data(), plan.classes.size() * sizeof(TileClass)));
+    CK(c, up(a.site, plan.site.data(), plan.site.size() * sizeof(int32_t)));
+    CK(c, up(a.orig, plan.orig.data(), plan.orig.size() * sizeof(int32_t)));
+    CK(c, up(a.halo_slot, plan.halo_slot.data(), plan.halo_slot.size() * sizeof(int32_t)));
+    CK(c, up(a.pub, plan.pub.data(), plan.pub.size() * sizeof(int32_t)));
+    CK(c, up(a.rows, plan.rows.get(), plan.row_bytes));
+    CK(c, up(a.codes, plan.codes.data(), plan.codes.size() * sizeof(float)));
+    CK(c, up(a.mail, nullptr, (size_t)plan.n_mail * c->R * sizeof(float4)));
+    CK(c, up(a.partial, nullptr, words * 4 * sizeof(double)));
+    CK(c, up(a.count, nullptr, words * sizeof(uint32_t)));
+    CK(c, up(a.abort, nullptr, sizeof(uint32_t)));
+    CK(c, cudaStreamSynchronize(c->stream));  // the plan goes out of scope
+    c->tile_ok = true;
+    return VEGAS_OK;
 }
 
 }  // namespace
@@ -1196,6 +1294,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         // (the resident sweep's, or built here), read without row offsets
         const int deg0 = c->passes[0].args.deg;
         bool use_ell = false;
+        if (!p64) TRY(make_tile(c, L[0]));
         if (!p64 && deg0 != 6) {
             int64_t max_deg = 0;
             for (int64_t g = 0; g < n_sites; ++g)
@@ -1395,6 +1494,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
             return bail(VEGAS_EINVAL);
         }
         c->variant = 2;
+        c->use_tile = c->tile_ok;
         c->tuned = true;
     } else if (o.variant == 3) {
         if (!c->cluster_eligible) {
@@ -1618,7 +1718,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             enqueue_coop(c, c->stream, n);
             if (c->opt.timing) CK(c, cudaEventRecord(ev[ev.size() - 1], c->stream));
             CK(c, cudaGetLastError());
-            c->kernel_launches += 2;
+            c->kernel_launches += coop_kernels(c, n);
             c->sweep_launches++;
             return VEGAS_OK;
         };
@@ -1755,6 +1855,22 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                         if (e4) break;  // report the device error below
                     }
                     c->variant = best_v;
+                    // The tiled form runs several times faster than any sweep timed above wherever it
+                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 29, 55; 32^3 x
+                    // 32 replicas 12, 38; the 29k-site core/shell particle 4.9, 23; a 13k-site fcc sphere
+                    // x 8 5.4, 24; 512 sites 2.1, 9), so it is not timed. It takes over where it adds the
+                    // attempts' FP32 shares in the order of the sweep that would run (one thread per
+                    // site of a class: the cooperative form, and every sweep of classes of at most 512
+                    // sites) or where that order is not fixed anyway (the kernel of 32 replicas draws its
+                    // blocks from a counter); elsewhere records would differ by the FP32 sums' rounding,
+                    // 1e-9 of their norm.
+                    if (c->tile_ok && !c->opt.resident_smem &&
+                        (best_v == 2 || c->max_class_sites <= kTileThreads ||
+                         (best_v == 0 && pass32_kind(c->passes[0].args) == VEGAS_KERNEL_PASS32_R32))) {
+                        c->variant = best_v = 2;
+                        best_c = Cand{2, 2, 0, 0, 0};
+                        c->use_tile = true;
+                    }
                     // the shape of the sweep kept goes last: the two persistent sweeps share the
                     // grouping of small instances
                     if (c->cluster_eligible && best_v != 3) set_cluster_shape(c, cs_rule, ct_rule, 0, 0, 0);
@@ -1781,7 +1897,9 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                     // reduction); or mcs x (passes + reduction)), the renormalisation, the snapshot,
                     // the loop control
                     const int64_t sweep_k = c->variant == 4 ? 2 * (int64_t)mcs
-                                            : (c->variant >= 1 ? 2 : (int64_t)mcs * ((int64_t)c->launches.size() + 1));
+                                            : (c->variant == 2   ? coop_kernels(c, mcs)
+                                               : c->variant >= 1 ? 2
+                                                                 : (int64_t)mcs * ((int64_t)c->launches.size() + 1));
                     c->kernel_launches += left * (sweep_k + (fold_active(c) ? 1 : 2) + (c->opt.snapshots ? 1 : 0));
                     c->sweep_launches += c->variant == 4 ? left * (int64_t)mcs
                                          : (c->variant >= 1 ? left : left * (int64_t)mcs * (int64_t)c->launches.size());
@@ -2140,6 +2258,7 @@ extern "C" vegas_status vegas_stats(const vegas_ctx *c, vegas_stats_t *o) {
         o->n_types = c->n_types;
         o->snapshot_steps = c->snapshot_steps;
         o->block_threads = c->variant == 1 ? c->res_threads : (c->variant == 3 ? c->cluster_threads : kThreads);
+        if (c->variant == 2 && c->use_tile) o->block_threads = c->tile_threads + kTileRecord;
         o->cluster_blocks = c->variant == 3 ? c->cluster_cs : 0;
         o->split_sites = c->variant == 3 ? c->res.split_sites : 0;
         o->group_threads = (c->variant == 1 || c->variant == 3) ? c->res.group_threads : 0;

@@ -105,7 +105,8 @@ __device__ __forceinline__ float3 trial_random32(uint4 rw, float sn) {
 // surrounding code. h is the exchange field sum_j J_ij S_j (row order), l its part over
 // lower colours (x and y of each as a packed pair: the packed FP32 instructions of sm_100+
 // round each lane as the scalar operation does, so the results are the same bits); wacc is
-// the random word of the acceptance uniform.
+// the random word of the acceptance uniform. PM: 0 no anisotropy, 1 and 2 both kinds, 3 uniaxial
+// only (the cubic terms of a zero constant change no bit: they are left out).
 template <int PM, int LM>
 __device__ __forceinline__ void attempt32(const float4 Si, float2 hxy, float hz, float2 lxy, float lz,
                                           const Site32 &p, float beta, float B, const float3 P, uint32_t wacc,
@@ -122,7 +123,7 @@ __device__ __forceinline__ void attempt32(const float4 Si, float2 hxy, float hz,
         const float pn = fmaf(px, p.ex, fmaf(py, p.ey, __fmul_rn(pz, p.ez)));
         const float po = fmaf(Si.x, p.ex, fmaf(Si.y, p.ey, __fmul_rn(Si.z, p.ez)));
         dE = fmaf(-p.k, __fmul_rn(__fsub_rn(pn, po), __fadd_rn(pn, po)), dE);
-        dE = fmaf(-p.kc, __fsub_rn(cub32(px, py, pz), cub32(Si.x, Si.y, Si.z)), dE);
+        if (PM != 3) dE = fmaf(-p.kc, __fsub_rn(cub32(px, py, pz), cub32(Si.x, Si.y, Si.z)), dE);
     }
     // Metropolis acceptance (Eq. 4) with the uniform u = wacc 2^-32 (all 32 random bits):
     // u < p  <=>  wacc < p 2^32, so the test is wacc < floor(p 2^32) (p 2^32 is exact in FP32,
@@ -139,7 +140,8 @@ __device__ __forceinline__ void attempt32(const float4 Si, float2 hxy, float hz,
     if (LM != 0) e = __fsub_rn(e, fmaf(qx, lx, fmaf(qy, ly, __fmul_rn(qz, lz))));
     if (PM != 0) {
         const float pe = fmaf(qx, p.ex, fmaf(qy, p.ey, __fmul_rn(qz, p.ez)));
-        e = __fsub_rn(e, fmaf(__fmul_rn(p.k, pe), pe, __fmul_rn(p.kc, cub32(qx, qy, qz))));
+        e = __fsub_rn(e, PM == 3 ? __fmul_rn(__fmul_rn(p.k, pe), pe)
+                                 : fmaf(__fmul_rn(p.k, pe), pe, __fmul_rn(p.kc, cub32(qx, qy, qz))));
     }
     e_i = e;
 }

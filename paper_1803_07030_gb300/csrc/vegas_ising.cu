@@ -81,7 +81,7 @@ __device__ __forceinline__ void append_reject(uint32_t &mask, uint32_t w, uint32
 // griddepcontrol.wait, so it overlaps the tail of the pass before (programmatic dependent
 // launch). S threads share a word position (32 / S sites each) on lattices too small to fill the
 // GPU. 960^2 x 32 replicas: 90 us per MCS with class look-ups and a reduction kernel of its own
-// (42 instructions per attempt), @@NOW@@ now.
+// (42 instructions per attempt), 27 us (1.08 T attempts/s) now.
 template <int DIMS, int NQ, int S>
 __global__ void __launch_bounds__(kIsingThreads) ising_pass_kernel(const IsingPassArgs a) {
     constexpr int Z = 2 * DIMS, NB = 32 / S;

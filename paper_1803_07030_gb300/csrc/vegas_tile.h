@@ -1,0 +1,86 @@
+// The tiled cooperative sweep (vegas_tile.cu): its plan, arguments and launcher.
+#pragma once
+
+#include <cstdint>
+#include <memory>
+#include <vector>
+
+#include "vegas_internal.h"
+
+namespace vegas {
+
+constexpr int kTileThreads = 512;     // most sweeping threads per block
+constexpr int kTileRecord = 128;      // threads of a block that form the MCS's totals
+constexpr int kTilePerClass = 64;     // at least so many sites of the widest class per part: finer parts
+                                      // only add boundary (29k-site core/shell particle, us per MCS: 4.9
+                                      // with 32 to 64, 5.2 with 96 or 128, 6.3 with 256)
+constexpr int kTileMcs = 1024;        // MCS per launch (bounds the buffer of the parts' totals)
+constexpr int kTileCodes = 32;        // most exchange values of rows kept as words
+constexpr int kTileRun = 64;          // most attempts of a thread per MCS (one FP32 run of its sums)
+
+struct TilePart {
+    int32_t own_begin, n_own;    // own sites: rows [own_begin, own_begin + n_own)
+    int32_t halo_begin, n_halo;  // remote sites it reads: words halo_slot[halo_begin ..)
+    int32_t site_begin;          // global sites of both, own first: site[site_begin ..)
+    int32_t word_begin, n_words; // mailbox words of its own sites
+};
+
+struct TileClass {               // one colour class of one part, local site numbers
+    int32_t begin, end;
+    int32_t halo_begin, halo_end;
+    int32_t lower_mode;          // 0: no link to a lower colour, 1: every link, 2: flagged per link
+};
+
+struct TileArgs {
+    PassArgs pass;
+    const TilePart *parts;       // [P]
+    const TileClass *classes;    // [P][n_colours]
+    const int32_t *site;         // global site of every local site of every part
+    const int32_t *orig;         // caller id of every own site
+    const int32_t *pub;          // mailbox word of every own site, -1 without a remote reader
+    const int32_t *halo_slot;    // mailbox word of every remote site of every part
+    const void *rows;            // [own site][width]: (local site | lower flag << 16, J) pairs, or words
+    const float *codes;          // [n_codes] exchange values of a sample whose rows are words
+    float4 *mail;                // [R][n_mail] (x, y, z, MCS counter + 1)
+    double *partial;             // [mcs][R][4][P]
+    uint32_t *count;             // [mcs][R][P] accepted attempts
+    uint32_t *abort;             // set when a wait ran out: every block leaves
+    int64_t timeout_ns;
+    uint32_t rk0[10], rk1[10];   // Philox round keys
+    int32_t P, n_colours, n_mail, mcs, width;
+    int32_t cubic;               // some site has a cubic constant
+    int32_t skip_block;          // fault injection: this block never runs (-1: none)
+    int32_t long_runs;           // threads take several attempts of a class: compensated sums
+    int32_t mem, n_codes, two_buffers;  // what is kept in shared memory (tile_shape)
+    int32_t cap, rows_off, orig_off, pub_off, slot_off, code_off, cls_off, part_off;  // and where
+};
+
+struct TileShape {               // a loaded sample (new numbering) and the parts to cut it into
+    int32_t n, n_colours, parts, width, site_off;
+    const int32_t *cstart, *lower_mode, *col, *orig;
+    const int64_t *row_ptr;
+    const double *J;
+};
+
+struct TilePlan {
+    std::vector<TilePart> parts;
+    std::vector<TileClass> classes;
+    std::vector<int32_t> site, orig, pub, halo_slot;
+    std::vector<int32_t> part, local, word; // of every site (word: from its part's first, -1: none)
+    std::vector<std::vector<int32_t>> own, halo;  // sites of every part
+    std::unique_ptr<unsigned char[]> rows;  // pairs or words (tile_shape)
+    size_t row_bytes = 0;
+    std::vector<float> codes;               // exchange values
+    int32_t n_mail = 0, max_own = 0, max_halo = 0, max_loc = 0, widest = 0;
+    bool columns = false;
+};
+
+// False when the sample cannot be cut so.
+bool tile_plan(const TileShape &s, TilePlan &out);
+// Chooses the threads per block and what it keeps in shared memory, and writes the rows; 0 when
+// the parts do not fit.
+int tile_shape(TileArgs &a, const TileShape &s, TilePlan &p, size_t *smem);
+// Sweep of a.mcs MCS and their records; returns the CUDA error.
+int launch_tile(const TileArgs &a, int threads, size_t smem, void *stream);
+
+}  // namespace vegas
