@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "vegas_exp64.cuh"
 #include "vegas_internal.h"
 
 using namespace vegas;
@@ -19,6 +20,7 @@ namespace {
 
 constexpr int kAnaThreads = 256;
 constexpr int kMaxObs = 8;  // observables per reweighting call
+constexpr int kMultiBatch = 16;  // fused reweighting iterations per host synchronisation
 
 thread_local std::string g_ana_err;
 
@@ -190,15 +192,24 @@ __global__ void __launch_bounds__(kAnaThreads) thermal_kernel(const double *seri
 }
 
 // ------------------------------------------------------------------ reweighting
+// Bound by FP64 issue (two operations per SM and clock), which the exponentials filled: every exp
+// is exp_int64 here, integer arithmetic only. tab: its table, copied into shared memory.
+__device__ __forceinline__ void load_exp_table(unsigned long long *tab) {
+    for (int k = threadIdx.x; k < 256; k += blockDim.x) tab[k] = kExp2Table[k];
+    __syncthreads();
+}
+
 // D_i = ln sum_j n exp(-beta_j E_i - g_j) for every sample i.
 __global__ void denom_kernel(const double *E, int64_t n_tot, const double *beta, const double *g, int32_t K,
                              double logn, double *D) {
+    __shared__ unsigned long long tab[256];
+    load_exp_table(tab);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_tot; i += (int64_t)gridDim.x * blockDim.x) {
         const double e = E[i];
         double m = -INFINITY;
         for (int j = 0; j < K; ++j) m = fmax(m, -beta[j] * e - g[j]);
         double s = 0.0;
-        for (int j = 0; j < K; ++j) s += exp(-beta[j] * e - g[j] - m);
+        for (int j = 0; j < K; ++j) s += exp_int64(-beta[j] * e - g[j] - m, tab);
         D[i] = logn + m + log(s);
     }
 }
@@ -209,11 +220,20 @@ __global__ void __launch_bounds__(kAnaThreads) lse_kernel(const double *E, const
                                                           int32_t n_obs, int64_t n_tot, const double *betas,
                                                           double *part) {
     __shared__ double sm[kAnaThreads / 32];
+    __shared__ unsigned long long tab[256];
+    load_exp_table(tab);
     const double beta = betas[blockIdx.y];
     const int64_t chunk = (n_tot + gridDim.x - 1) / gridDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = min(n_tot, i0 + chunk);
-    double m = -INFINITY;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) m = fmax(m, -beta * E[i] - D[i]);
+    // the maximum by integer comparisons of the values' bits (mapped so that their order is the
+    // values'): a comparison of doubles is an FP64 instruction
+    auto ordered = [](long long v) { return v ^ ((v >> 63) & 0x7FFFFFFFFFFFFFFFLL); };
+    long long mk = ordered(__double_as_longlong(-INFINITY));
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+        const long long v = __double_as_longlong(-beta * E[i] - D[i]);
+        if ((v & 0x7FFFFFFFFFFFFFFFLL) <= 0x7FF0000000000000LL) mk = max(mk, ordered(v));  // not NaN
+    }
+    double m = __longlong_as_double(ordered(mk));
     // block max (fixed order)
     for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
     __shared__ double smax[kAnaThreads / 32];
@@ -222,58 +242,201 @@ __global__ void __launch_bounds__(kAnaThreads) lse_kernel(const double *E, const
     double M = -INFINITY;
     for (int w = 0; w < kAnaThreads / 32; ++w) M = fmax(M, smax[w]);
     double s = 0.0, so[kMaxObs];
+#pragma unroll
     for (int q = 0; q < kMaxObs; ++q) so[q] = 0.0;
     if (M > -INFINITY) {
         for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-            const double w = exp(-beta * E[i] - D[i] - M);
+            const double w = exp_int64(-beta * E[i] - D[i] - M, tab);
             s += w;
-            for (int q = 0; q < n_obs; ++q) so[q] += w * O[i * n_obs + q];
+#pragma unroll
+            for (int q = 0; q < kMaxObs; ++q)
+                if (q < n_obs) so[q] += w * O[i * n_obs + q];
         }
     }
     double *p = part + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (2 + kMaxObs);
     const double ts = block_sum(s, sm);
     double to[kMaxObs];
-    for (int q = 0; q < n_obs; ++q) to[q] = block_sum(so[q], sm);
+#pragma unroll
+    for (int q = 0; q < kMaxObs; ++q)
+        if (q < n_obs) to[q] = block_sum(so[q], sm);
     if (threadIdx.x == 0) {
         p[0] = M;
         p[1] = ts;
-        for (int q = 0; q < n_obs; ++q) p[2 + q] = to[q];
+#pragma unroll
+        for (int q = 0; q < kMaxObs; ++q)
+            if (q < n_obs) p[2 + q] = to[q];
     }
 }
 
-// Combines the per-block partials of each row y in block order: lse[y] = M + ln S and, when
-// obs is not NULL, obs[y][q] = sum O exp(x) / sum exp(x).
+// Combines the per-block partials of each row y, one warp per row (lanes over the blocks, then a
+// butterfly): lse[y] = M + ln S and, when obs is not NULL, obs[y][q] = sum O exp(x) / sum exp(x).
 __global__ void combine_kernel(const double *part, int32_t n_parts, int32_t n_rows, int32_t n_obs, double *lse,
                                double *obs) {
-    const int y = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (y >= n_rows) return;
     const double *p = part + (int64_t)y * n_parts * (2 + kMaxObs);
     double M = -INFINITY;
-    for (int b = 0; b < n_parts; ++b) M = fmax(M, p[b * (2 + kMaxObs)]);
+    for (int b = lane; b < n_parts; b += 32) M = fmax(M, p[b * (2 + kMaxObs)]);
+    for (int off = 16; off > 0; off >>= 1) M = fmax(M, __shfl_xor_sync(0xFFFFFFFFu, M, off));
     double s = 0.0, so[kMaxObs];
+#pragma unroll
     for (int q = 0; q < kMaxObs; ++q) so[q] = 0.0;
-    for (int b = 0; b < n_parts; ++b) {
+    for (int b = lane; b < n_parts; b += 32) {
         const double *pb = p + b * (2 + kMaxObs);
         if (pb[0] == -INFINITY) continue;
         const double f = exp(pb[0] - M);
         s += pb[1] * f;
-        for (int q = 0; q < n_obs; ++q) so[q] += pb[2 + q] * f;
+#pragma unroll
+        for (int q = 0; q < kMaxObs; ++q)
+            if (q < n_obs) so[q] += pb[2 + q] * f;
     }
+    for (int off = 16; off > 0; off >>= 1) {
+        s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+#pragma unroll
+        for (int q = 0; q < kMaxObs; ++q)
+            if (q < n_obs) so[q] += __shfl_xor_sync(0xFFFFFFFFu, so[q], off);
+    }
+    if (lane != 0) return;
     lse[y] = M + log(s);
     if (obs)
-        for (int q = 0; q < n_obs; ++q) obs[(int64_t)y * n_obs + q] = so[q] / s;
+#pragma unroll
+        for (int q = 0; q < kMaxObs; ++q)
+            if (q < n_obs) obs[(int64_t)y * n_obs + q] = so[q] / s;
 }
 
-struct DevBuf {
-    std::vector<void *> ptrs;
-    ~DevBuf() {
-        for (void *p : ptrs) cudaFree(p);
+// State of the fixed-point iteration g_j <- ln sum_i exp(-beta_j E_i - D_i(g)), on the device.
+struct MultiState {
+    double diff;
+    int32_t iters;    // iterations done
+    uint32_t ticket;  // blocks done in the current one
+    int32_t stop;     // 1: diff < tol, 2: a step the fused form cannot take (nothing was changed)
+};
+
+constexpr int kMultiRuns = 16;  // most runs of the fused form (a thread keeps two values per run)
+
+// One iteration in one launch, for at most KM runs. With z_ij = -beta_j E_i - g_j the sample's
+// denominator is n sum_j exp(z_ij), and the new g_j = g_j + ln sum_i a_ij / s_i - ln n with
+// a_ij = exp(z_ij - z_ik), s_i = sum_j a_ij, k the sample's own run: the same K exponentials give
+// the denominators and the sums, so none is taken twice and no logarithm per sample is left.
+// A block takes a range of one run's samples (so z_ij - z_ik = db_j E_i + dg_j with its own few
+// constants) and the last block combines the blocks' sums. Three FP64 operations per
+// exponential and seven per sample remain. Values that leave the range of exp_int64, or a sum that
+// underflows, stop the iteration unchanged (stop = 2) and the kernels above take that step.
+// 8 runs x 20,011 samples: 364 us per iteration before (denom, lse and combine kernels with FP64
+// exponentials, and a host synchronisation), 22.5 us now (half of it the FP64 pipe's share).
+template <int KM>
+__global__ void __launch_bounds__(kAnaThreads) multi_step_kernel(const double *E, int64_t n, int32_t K, const double *beta,
+                                                                 double *g, double logn, double tol, double *part,
+                                                                 MultiState *st) {
+    __shared__ unsigned long long tab[256];
+    __shared__ double s_db[KM], s_dg[KM];
+    __shared__ double s_sum[KM][kAnaThreads + 8];
+    __shared__ bool s_last;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int k = blockIdx.y, tid = threadIdx.x;
+    for (int q = tid; q < 256; q += kAnaThreads) tab[q] = kExp2Table[q];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (__ldcg(&st->stop) != 0) return;
+    if (tid < KM) {
+        s_db[tid] = tid < K ? beta[k] - beta[tid] : 0.0;
+        s_dg[tid] = tid < K ? __ldcg(g + k) - __ldcg(g + tid) : 0.0;
     }
+    __syncthreads();
+    double P[KM];
+#pragma unroll
+    for (int j = 0; j < KM; ++j) P[j] = 0.0;
+    const int64_t chunk = (n + gridDim.x - 1) / gridDim.x, i0 = (int64_t)blockIdx.x * chunk, i1 = min(n, i0 + chunk);
+    for (int64_t i = i0 + tid; i < i1; i += kAnaThreads) {
+        const double e = E[(int64_t)k * n + i];
+        double a[KM], s = 0.0;
+#pragma unroll
+        for (int j = 0; j < KM; ++j) {
+            a[j] = 0.0;
+            if (j < K) {
+                a[j] = exp_int64(fma(s_db[j], e, s_dg[j]), tab);
+                s += a[j];
+            }
+        }
+        // 1 / s by Newton's iteration on the hardware's approximation (s >= 1; an infinite s leaves NaN)
+        double r;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s));
+        r = fma(r, fma(-s, r, 1.0), r);
+        r = fma(r, fma(-s, r, 1.0), r);
+#pragma unroll
+        for (int j = 0; j < KM; ++j)
+            if (j < K) P[j] = fma(a[j], r, P[j]);
+    }
+    // block sums with few FP64 instructions: threads' values through shared memory, kAnaThreads / KM
+    // lanes per run adding KM each, then a butterfly over those lanes
+    constexpr int L = kAnaThreads / KM;
+#pragma unroll
+    for (int j = 0; j < KM; ++j) s_sum[j][tid] = P[j];
+    __syncthreads();
+    {
+        const int j = tid / L, l = tid % L;
+        double v = 0.0;
+        for (int q = l; q < kAnaThreads; q += L) v += s_sum[j][q];
+        for (int off = (L < 32 ? L : 32) / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        __syncthreads();
+        if (l % 32 == 0) s_sum[j][l / 32] = v;
+        __syncthreads();
+        if (tid < KM && tid < K) {
+            double t = s_sum[tid][0];
+            for (int q = 1; q < (L + 31) / 32; ++q) t += s_sum[tid][q];
+            part[((int64_t)k * gridDim.x + blockIdx.x) * KM + tid] = t;
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&st->ticket, 1u) == gridDim.x * gridDim.y - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // the last block: one warp per run adds the blocks' sums in order (lanes striding, a butterfly)
+    const int n_part = gridDim.x * gridDim.y, lane = tid & 31;
+    for (int j = tid >> 5; j < K; j += kAnaThreads / 32) {
+        double v = 0.0;
+        for (int b = lane; b < n_part; b += 32) v += __ldcg(part + (int64_t)b * KM + j);
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        if (lane == 0) s_sum[0][j] = v;
+    }
+    __syncthreads();
+    if (tid < 32) {  // one lane per run (KM <= 16)
+        const double sum = lane < K ? s_sum[0][lane] : 1.0, old = lane < K ? __ldcg(g + lane) : 0.0;
+        const bool fine = sum > 1e-200 && sum < 1e200;
+        double v = old + (log(sum) - logn);
+        v -= __shfl_sync(0xFFFFFFFFu, v, 0);  // gauge: g_0 = 0
+        double d = lane < K ? fabs(v - old) : 0.0;
+        for (int off = 16; off > 0; off >>= 1) d = fmax(d, __shfl_xor_sync(0xFFFFFFFFu, d, off));
+        const bool all = __all_sync(0xFFFFFFFFu, fine);
+        if (all && lane < K) g[lane] = v;
+        if (lane == 0) {
+            st->ticket = 0;
+            if (all) {
+                st->diff = d;
+                st->iters += 1;
+            }
+            st->stop = !all ? 2 : (d < tol ? 1 : 0);
+        }
+    }
+}
+
+// Device memory of one call: one allocation cut into 256-byte aligned pieces (an allocation and its
+// release take about 20 us each). reserve() every piece, then allocate(), then take() them in order.
+struct DevBuf {
+    char *base = nullptr;
+    size_t size = 0, used = 0;
+    ~DevBuf() {
+        if (base) cudaFree(base);
+    }
+    static size_t padded(size_t bytes) { return (bytes + 255) / 256 * 256; }
+    void reserve(size_t bytes) { size += padded(bytes); }
+    cudaError_t allocate() { return cudaMalloc((void **)&base, size > 0 ? size : 256); }
     template <typename T>
-    cudaError_t alloc(T **p, size_t bytes) {
-        cudaError_t e = cudaMalloc((void **)p, bytes > 0 ? bytes : 8);
-        if (e == cudaSuccess) ptrs.push_back(*p);
-        return e;
+    T *take(size_t bytes) {
+        T *p = (T *)(base + used);
+        used += padded(bytes);
+        return p;
     }
 };
 
@@ -311,13 +474,12 @@ extern "C" vegas_status vegas_thermal_averages(const double *series, int64_t n_s
         vegas_status st = have_device();
         if (st != VEGAS_OK) return st;
         cudaStream_t stream = (cudaStream_t)cuda_stream;
-        DevBuf b;
-        double *d_h, *d_T, *d_N, *d_out;
         const size_t hb = sizeof(double) * 4 * (size_t)n_series * (size_t)len;
-        ACK(b.alloc(&d_h, hb));
-        ACK(b.alloc(&d_T, sizeof(double) * n_series));
-        ACK(b.alloc(&d_N, sizeof(double) * n_series));
-        ACK(b.alloc(&d_out, sizeof(double) * VEGAS_AVG_FIELDS * n_series));
+        const size_t sb = sizeof(double) * (size_t)n_series, ob = VEGAS_AVG_FIELDS * sb;
+        DevBuf b;
+        for (const size_t x : {hb, sb, sb, ob}) b.reserve(x);
+        ACK(b.allocate());
+        double *d_h = b.take<double>(hb), *d_T = b.take<double>(sb), *d_N = b.take<double>(sb), *d_out = b.take<double>(ob);
         ACK(cudaMemcpyAsync(d_h, series, hb, cudaMemcpyHostToDevice, stream));
         ACK(cudaMemcpyAsync(d_T, T, sizeof(double) * n_series, cudaMemcpyHostToDevice, stream));
         ACK(cudaMemcpyAsync(d_N, n_sites, sizeof(double) * n_series, cudaMemcpyHostToDevice, stream));
@@ -343,24 +505,35 @@ extern "C" vegas_status vegas_reweight(const double *E, const double *O, int32_t
         const int64_t n_tot = (int64_t)K * n;
         for (int32_t k = 0; k < K; ++k)
             if (!std::isfinite(betas_k[k])) return ana_fail(VEGAS_EINVAL, "non-finite beta");
-        for (int64_t i = 0; i < n_tot; ++i)
-            if (!std::isfinite(E[i])) return ana_fail(VEGAS_EINVAL, "non-finite energy");
+        int bad = 0;  // no early exit: the loop vectorises
+        for (int64_t i = 0; i < n_tot; ++i) bad |= !(std::fabs(E[i]) <= 1.7976931348623157e308);
+        if (bad) return ana_fail(VEGAS_EINVAL, "non-finite energy");
         vegas_status st = have_device();
         if (st != VEGAS_OK) return st;
         cudaStream_t stream = (cudaStream_t)cuda_stream;
-        DevBuf b;
-        double *d_E, *d_O, *d_D, *d_bk, *d_bo, *d_g, *d_lse, *d_part, *d_obs;
+        int dev = 0, sms = 1;
+        ACK(cudaGetDevice(&dev));
+        ACK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const int parts = (int)std::min<int64_t>(256, (n_tot + kAnaThreads - 1) / kAnaThreads);
+        // the averages' rows fill the GPU together: about eight blocks per SM over all of them, so that a
+        // thread has many samples to a block sum (40 rows of 160,000: 540 us with 256 blocks per row)
+        const int parts_out = std::max(1, std::min(parts, 8 * sms / std::max(n_out, 1)));
         const int rows = std::max<int32_t>(K, n_out);
-        ACK(b.alloc(&d_E, sizeof(double) * n_tot));
-        ACK(b.alloc(&d_O, sizeof(double) * n_tot * std::max(n_obs, 1)));
-        ACK(b.alloc(&d_D, sizeof(double) * n_tot));
-        ACK(b.alloc(&d_bk, sizeof(double) * K));
-        ACK(b.alloc(&d_bo, sizeof(double) * std::max(n_out, 1)));
-        ACK(b.alloc(&d_g, sizeof(double) * K));
-        ACK(b.alloc(&d_lse, sizeof(double) * rows));
-        ACK(b.alloc(&d_part, sizeof(double) * (2 + kMaxObs) * (size_t)parts * rows));
-        ACK(b.alloc(&d_obs, sizeof(double) * (size_t)std::max(n_out, 1) * std::max(n_obs, 1)));
+        // fused iterations: two blocks per SM over all runs, at least kAnaThreads samples each
+        const bool fused = K <= kMultiRuns;
+        const int mx = (int)std::max<int64_t>(1, std::min<int64_t>(2 * sms / K, (n + kAnaThreads - 1) / kAnaThreads));
+        const size_t D = sizeof(double), nb = D * (size_t)n_tot, kb = D * (size_t)K, tb = D * (size_t)std::max(n_out, 1);
+        const size_t pb = D * std::max<size_t>((size_t)(2 + kMaxObs) * parts * rows, (size_t)mx * K * kMultiRuns);
+        DevBuf b;
+        for (const size_t x : {nb, nb * std::max(n_obs, 1), nb, kb, tb, kb, D * (size_t)rows, pb, tb * std::max(n_obs, 1),
+                               sizeof(MultiState)})
+            b.reserve(x);
+        ACK(b.allocate());
+        double *d_E = b.take<double>(nb), *d_O = b.take<double>(nb * std::max(n_obs, 1)), *d_D = b.take<double>(nb);
+        double *d_bk = b.take<double>(kb), *d_bo = b.take<double>(tb), *d_g = b.take<double>(kb);
+        double *d_lse = b.take<double>(D * (size_t)rows), *d_part = b.take<double>(pb);
+        double *d_obs = b.take<double>(tb * std::max(n_obs, 1));
+        MultiState *d_st = b.take<MultiState>(sizeof(MultiState));
         ACK(cudaMemcpyAsync(d_E, E, sizeof(double) * n_tot, cudaMemcpyHostToDevice, stream));
         if (n_obs > 0) ACK(cudaMemcpyAsync(d_O, O, sizeof(double) * n_tot * n_obs, cudaMemcpyHostToDevice, stream));
         ACK(cudaMemcpyAsync(d_bk, betas_k, sizeof(double) * K, cudaMemcpyHostToDevice, stream));
@@ -369,32 +542,75 @@ extern "C" vegas_status vegas_reweight(const double *E, const double *O, int32_t
         ACK(cudaMemcpyAsync(d_g, g.data(), sizeof(double) * K, cudaMemcpyHostToDevice, stream));
         const double logn = std::log((double)n);
         const int dgrid = (int)std::min<int64_t>((n_tot + 255) / 256, 4096);
-        int32_t it = 0;
-        for (it = 1; it <= max_iter; ++it) {
-            denom_kernel<<<dgrid, 256, 0, stream>>>(d_E, n_tot, d_bk, d_g, K, logn, d_D);
-            lse_kernel<<<dim3(parts, K), kAnaThreads, 0, stream>>>(d_E, d_D, d_O, 0, n_tot, d_bk, d_part);
-            combine_kernel<<<(K + 127) / 128, 128, 0, stream>>>(d_part, parts, K, 0, d_lse, nullptr);
-            ACK(cudaGetLastError());
-            ACK(cudaMemcpyAsync(gn.data(), d_lse, sizeof(double) * K, cudaMemcpyDeviceToHost, stream));
-            ACK(cudaStreamSynchronize(stream));
-            double diff = 0.0;
-            const double g0 = gn[0];
-            for (int32_t k = 0; k < K; ++k) {
-                gn[(size_t)k] -= g0;  // gauge: g_0 = 0
-                diff = std::max(diff, std::fabs(gn[(size_t)k] - g[(size_t)k]));
+        auto combine = [&](int n_parts, int n_rows, int obs_, double *d_o) {
+            combine_kernel<<<(n_rows + 3) / 4, 128, 0, stream>>>(d_part, n_parts, n_rows, obs_, d_lse, d_o);
+        };
+        MultiState ms{};
+        ACK(cudaMemcpyAsync(d_st, &ms, sizeof ms, cudaMemcpyHostToDevice, stream));
+        int32_t it = 0;  // iterations done
+        bool done = false, general = !fused;
+        while (!done && it < max_iter) {
+            if (general) {  // one iteration by the separate kernels
+                denom_kernel<<<dgrid, 256, 0, stream>>>(d_E, n_tot, d_bk, d_g, K, logn, d_D);
+                lse_kernel<<<dim3(parts, K), kAnaThreads, 0, stream>>>(d_E, d_D, d_O, 0, n_tot, d_bk, d_part);
+                combine(parts, K, 0, nullptr);
+                ACK(cudaGetLastError());
+                ACK(cudaMemcpyAsync(gn.data(), d_lse, sizeof(double) * K, cudaMemcpyDeviceToHost, stream));
+                ACK(cudaStreamSynchronize(stream));
+                double diff = 0.0;
+                const double g0 = gn[0];
+                for (int32_t k = 0; k < K; ++k) {
+                    gn[(size_t)k] -= g0;  // gauge: g_0 = 0
+                    diff = std::max(diff, std::fabs(gn[(size_t)k] - g[(size_t)k]));
+                }
+                if (!std::isfinite(diff))
+                    return ana_fail(VEGAS_EDEVICE, "reweighting iteration produced a non-finite value");
+                g = gn;
+                ACK(cudaMemcpyAsync(d_g, g.data(), sizeof(double) * K, cudaMemcpyHostToDevice, stream));
+                ++it;
+                done = diff < tol;
+                general = !fused;
+                continue;
             }
-            g = gn;
-            ACK(cudaMemcpyAsync(d_g, g.data(), sizeof(double) * K, cudaMemcpyHostToDevice, stream));
-            if (!std::isfinite(diff)) return ana_fail(VEGAS_EDEVICE, "reweighting iteration produced a non-finite value");
-            if (diff < tol) break;
+            // a batch of fused iterations; those after the last one needed return at once
+            ms = MultiState{0.0, it, 0u, 0};
+            ACK(cudaMemcpyAsync(d_st, &ms, sizeof ms, cudaMemcpyHostToDevice, stream));
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)mx, (unsigned)K);
+            cfg.blockDim = dim3(kAnaThreads);
+            cfg.stream = stream;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            const int batch = (int)std::min<int64_t>(kMultiBatch, max_iter - it);
+            for (int q = 0; q < batch; ++q) {
+                if (K <= 4)
+                    ACK(cudaLaunchKernelEx(&cfg, multi_step_kernel<4>, (const double *)d_E, n, K, (const double *)d_bk, d_g,
+                                           logn, tol, d_part, d_st));
+                else if (K <= 8)
+                    ACK(cudaLaunchKernelEx(&cfg, multi_step_kernel<8>, (const double *)d_E, n, K, (const double *)d_bk, d_g,
+                                           logn, tol, d_part, d_st));
+                else
+                    ACK(cudaLaunchKernelEx(&cfg, multi_step_kernel<16>, (const double *)d_E, n, K, (const double *)d_bk, d_g,
+                                           logn, tol, d_part, d_st));
+            }
+            ACK(cudaMemcpyAsync(&ms, d_st, sizeof ms, cudaMemcpyDeviceToHost, stream));
+            ACK(cudaMemcpyAsync(g.data(), d_g, sizeof(double) * K, cudaMemcpyDeviceToHost, stream));
+            ACK(cudaStreamSynchronize(stream));
+            it = ms.iters;
+            done = ms.stop == 1;
+            general = ms.stop == 2;
+            if (it > 0 && !general && !std::isfinite(ms.diff))
+                return ana_fail(VEGAS_EDEVICE, "reweighting iteration produced a non-finite value");
         }
-        if (it > max_iter) it = max_iter;
         if (g_out) std::memcpy(g_out, g.data(), sizeof(double) * K);
         if (iters_out) *iters_out = it;
         if (n_out > 0) {
             denom_kernel<<<dgrid, 256, 0, stream>>>(d_E, n_tot, d_bk, d_g, K, logn, d_D);
-            lse_kernel<<<dim3(parts, n_out), kAnaThreads, 0, stream>>>(d_E, d_D, d_O, n_obs, n_tot, d_bo, d_part);
-            combine_kernel<<<(n_out + 127) / 128, 128, 0, stream>>>(d_part, parts, n_out, n_obs, d_lse, d_obs);
+            lse_kernel<<<dim3(parts_out, n_out), kAnaThreads, 0, stream>>>(d_E, d_D, d_O, n_obs, n_tot, d_bo, d_part);
+            combine(parts_out, n_out, n_obs, d_obs);
             ACK(cudaGetLastError());
             if (n_obs > 0)
                 ACK(cudaMemcpyAsync(out, d_obs, sizeof(double) * n_out * n_obs, cudaMemcpyDeviceToHost, stream));
