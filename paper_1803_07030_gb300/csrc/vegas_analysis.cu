@@ -3,6 +3,7 @@
 // (Sec. II, Sec. IV.A-B), and single/multiple histogram reweighting (Sec. IV.E; Ferrenberg
 // & Swendsen 1988, 1989). FP64 throughout; every sum is a fixed-order block reduction, so
 // results do not change between runs.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -48,147 +49,260 @@ __device__ double block_sum(double v, double *sm) {
     return s;
 }
 
-// Sums over records [i0, i1) of one series: the eight shifted moments
-//   e' = E - Eref, a' = |M| - Aref:  e', e'^2, a', a'^2, a' e', M^2, M^4, M^2 e'.
-__device__ void moment_sums(const double *h, int64_t i0, int64_t i1, double Eref, double Aref, double *sm,
-                            double out[8]) {
+// Sums over the block of the NQ values of every thread, in a fixed order, into out (shared memory),
+// with few FP64 instructions (an FP64 instruction of a warp takes 64 cycles here, whatever its
+// lanes do): warp w adds the threads' quantities w, w + 8, ... (a stride per lane, then a butterfly).
+template <int NQ>
+__device__ __forceinline__ void block_sums(const double (&v)[NQ], double (*sm)[kAnaThreads], double *out) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) sm[q][threadIdx.x] = v[q];
+    __syncthreads();
+    for (int q = threadIdx.x >> 5; q < NQ; q += kAnaThreads / 32) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < kAnaThreads / 32; ++k) s += sm[q][lane + 32 * k];
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+        if (lane == 0) out[q] = s;
+    }
+    __syncthreads();
+}
+
+// Thermal averages run as four kernels over all series: |M| and the plain sums; centred values and
+// moments per bin; estimates and errors; autocorrelation times. (One block per series with every
+// step inside, |M| taken anew for every lag and the errors on one thread, took 4.4 ms for 64 series of
+// 10,007 records, on 64 SMs and bound by their FP64 pipes; the whole call, with the 20 MB of records
+// copied from the host, went from 5.1 to 0.59 ms.)
+struct ThermalArgs {
+    const double *series;  // [n_series][len][4]
+    double *x;             // [2][n_series][stride]: E and |M| after the cut, then centred; zeros behind
+    double *sums;          // [n_series][chunks][2]
+    double *bins;          // [n_series][n_bins + 1][8], the last of the records behind the bins
+    const double *T, *Nsites;
+    double *out;           // [n_series][VEGAS_AVG_FIELDS]
+    int64_t len, cut, n, stride, chunk;
+    int32_t n_series, n_bins, chunks;
+};
+
+// |M| of every record after the cut, kept with E, and their sums over a chunk.
+__global__ void __launch_bounds__(kAnaThreads) thermal_load_kernel(const ThermalArgs a) {
+    __shared__ double sm[2][kAnaThreads], s_out[2];
+    const int64_t sid = blockIdx.y;
+    const double *h = a.series + (sid * a.len + a.cut) * 4;
+    double *xe = a.x + sid * a.stride, *xa = a.x + (a.n_series + sid) * a.stride;
+    const int64_t i0 = blockIdx.x * a.chunk, i1 = min(a.n, i0 + a.chunk);
+    double v[2] = {0.0, 0.0};
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kAnaThreads) {
+        const double2 p = ((const double2 *)h)[2 * i], q = ((const double2 *)h)[2 * i + 1];
+        const double m = sqrt(p.y * p.y + q.x * q.x + q.y * q.y);
+        xe[i] = p.x;
+        xa[i] = m;
+        v[0] += p.x;
+        v[1] += m;
+    }
+    block_sums<2>(v, sm, s_out);
+    if (threadIdx.x < 2) a.sums[(sid * a.chunks + blockIdx.x) * 2 + threadIdx.x] = s_out[threadIdx.x];
+}
+
+// Mean of E and |M| over a series (the same in every block that asks).
+__device__ __forceinline__ void series_means(const ThermalArgs &a, int64_t sid, double &Eref, double &Aref) {
+    double v[2] = {0.0, 0.0};
+    for (int k = threadIdx.x & 31; k < a.chunks; k += 32) {
+        v[0] += a.sums[(sid * a.chunks + k) * 2];
+        v[1] += a.sums[(sid * a.chunks + k) * 2 + 1];
+    }
+    for (int off = 16; off > 0; off >>= 1)
+        for (int q = 0; q < 2; ++q) v[q] += __shfl_xor_sync(0xFFFFFFFFu, v[q], off);
+    Eref = v[0] / (double)a.n;
+    Aref = v[1] / (double)a.n;
+}
+
+// Centred values e' = E - Eref, a' = |M| - Aref of one bin (block n_bins: the records behind the
+// bins), in place, and their moments: sums of e', e'^2, a', a'^2, a' e', M^2, M^4, M^2 e'.
+__global__ void __launch_bounds__(kAnaThreads) thermal_bin_kernel(const ThermalArgs a) {
+    __shared__ double sm[8][kAnaThreads], s_out[8], s_ref[2];
+    const int64_t sid = blockIdx.y, b = a.n / a.n_bins;
+    if (threadIdx.x < 32) {
+        double e, m;
+        series_means(a, sid, e, m);
+        if (threadIdx.x == 0) {
+            s_ref[0] = e;
+            s_ref[1] = m;
+        }
+    }
+    __syncthreads();
+    const double Eref = s_ref[0], Aref = s_ref[1];
+    double *xe = a.x + sid * a.stride, *xa = a.x + (a.n_series + sid) * a.stride;
+    const bool rest = (int)blockIdx.x == a.n_bins;
+    const int64_t i0 = blockIdx.x * b, i1 = rest ? a.n : i0 + b;
     double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        const double *r = h + i * 4;
-        const double m2 = r[1] * r[1] + r[2] * r[2] + r[3] * r[3];
-        const double e = r[0] - Eref, a = sqrt(m2) - Aref;
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kAnaThreads) {
+        const double m = xa[i], m2 = m * m, e = xe[i] - Eref, d = m - Aref;
+        xe[i] = e;
+        xa[i] = d;
         v[0] += e;
         v[1] += e * e;
-        v[2] += a;
-        v[3] += a * a;
-        v[4] += a * e;
+        v[2] += d;
+        v[3] += d * d;
+        v[4] += d * e;
         v[5] += m2;
         v[6] += m2 * m2;
         v[7] += m2 * e;
     }
-    for (int q = 0; q < 8; ++q) out[q] = block_sum(v[q], sm);
+    if (rest)  // zeros behind the series: the lags read past its end
+        for (int64_t i = a.n + threadIdx.x; i < a.stride; i += kAnaThreads) xe[i] = xa[i] = 0.0;
+    block_sums<8>(v, sm, s_out);
+    if (threadIdx.x < 8) a.bins[(sid * (a.n_bins + 1) + blockIdx.x) * 8 + threadIdx.x] = s_out[threadIdx.x];
 }
 
 // (c, chi, u4) from moment sums over n samples.
-__device__ void estimates(const double S[8], double n, double N, double T, double out[3]) {
+__device__ __forceinline__ void estimates(const double (&S)[8], double n, double N, double T, double (&out)[3]) {
     const double me = S[0] / n, ma = S[2] / n, m2 = S[5] / n;
     out[0] = (S[1] / n - me * me) / (N * T * T);
     out[1] = (S[3] / n - ma * ma) / (N * T);
     out[2] = 1.0 - (S[6] / n) / (3.0 * m2 * m2);
 }
 
-// Integrated autocorrelation time of x_i = (E or |M|) - mean, Sokal's window (c = 6).
-__device__ double tau_window(const double *h, int64_t cut, int64_t n, int which, double mean, double *sm) {
-    auto x = [&](int64_t i) {
-        const double *r = h + (cut + i) * 4;
-        return (which == 0 ? r[0] : sqrt(r[1] * r[1] + r[2] * r[2] + r[3] * r[3])) - mean;
-    };
-    double c0 = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const double d = x(i);
-        c0 += d * d;
-    }
-    c0 = block_sum(c0, sm) / (double)n;
-    if (c0 == 0.0) return 0.5;
-    double tau = 0.5;
-    for (int64_t t = 1; t <= n / 2; ++t) {
-        double c = 0.0;
-        for (int64_t i = threadIdx.x; i < n - t; i += blockDim.x) c += x(i) * x(i + t);
-        c = block_sum(c, sm) / (double)(n - t);
-        tau += c / c0;
-        if ((double)t >= 6.0 * tau) break;
-    }
-    return tau;
+__device__ __forceinline__ double warp_sum(double v) {
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+    return v;
 }
 
-// One block per series: point estimates over all records after the cut, errors from n_bins
-// equal bins over the first b * n_bins of them.
-__global__ void __launch_bounds__(kAnaThreads) thermal_kernel(const double *series, int64_t len, int64_t cut,
-                                                              int32_t n_bins, const double *T, const double *Nsites,
-                                                              double *out) {
-    __shared__ double sm[kAnaThreads / 32];
-    __shared__ double s_bin[64][8];  // n_bins <= 64
+// Point estimates over all records after the cut, errors from n_bins <= 64 equal bins (their spread
+// and leave-one-bin-out jackknife estimates): one warp per series, a lane takes bins lane, lane + 32.
+__global__ void thermal_estimate_kernel(const ThermalArgs a) {
     const int64_t sid = blockIdx.x;
-    const double *h = series + sid * len * 4;
-    const int64_t n = len - cut;
-    const double Tt = T[sid], N = Nsites[sid];
-    // reference shifts: the plain means of E and |M|
-    double s0 = 0.0, s1 = 0.0;
-    for (int64_t i = cut + threadIdx.x; i < len; i += blockDim.x) {
-        const double *r = h + i * 4;
-        s0 += r[0];
-        s1 += sqrt(r[1] * r[1] + r[2] * r[2] + r[3] * r[3]);
+    const int lane = threadIdx.x;
+    const double *bins = a.bins + sid * (a.n_bins + 1) * 8;
+    const double dn = (double)a.n, N = a.Nsites[sid], T = a.T[sid], nb = (double)a.n_bins;
+    const double db = (double)(a.n / a.n_bins);
+    double Eref, Aref;
+    series_means(a, sid, Eref, Aref);
+    double tot = 0.0;  // lane q < 8: quantity q over the bins
+    if (lane < 8)
+        for (int k = 0; k < a.n_bins; ++k) tot += bins[k * 8 + lane];
+    const double all = lane < 8 ? tot + bins[a.n_bins * 8 + lane] : 0.0;
+    double Tot[8], S[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        Tot[q] = __shfl_sync(0xFFFFFFFFu, tot, q);
+        S[q] = __shfl_sync(0xFFFFFFFFu, all, q);
     }
-    const double Eref = block_sum(s0, sm) / (double)n;
-    const double Aref = block_sum(s1, sm) / (double)n;
-    double S[8];
-    moment_sums(h, cut, len, Eref, Aref, sm, S);
-    const int64_t b = n / n_bins;
-    for (int k = 0; k < n_bins; ++k) {
-        double Sk[8];
-        moment_sums(h, cut + k * b, cut + (k + 1) * b, Eref, Aref, sm, Sk);
-        if (threadIdx.x == 0)
-            for (int q = 0; q < 8; ++q) s_bin[k][q] = Sk[q];
-    }
-    const double dn = (double)n;
-    const double meanE = Eref + S[0] / dn, meanA = Aref + S[2] / dn, meanM2 = S[5] / dn;
-    const double tau_e = tau_window(h, cut, n, 0, meanE, sm);
-    const double tau_m = tau_window(h, cut, n, 1, meanA, sm);
-    if (threadIdx.x != 0) return;
+    const double de = S[0] / dn, da = S[2] / dn, meanE = Eref + de, meanA = Aref + da, meanM2 = S[5] / dn;
     double est[3];
-    estimates(S, dn, N, Tt, est);
-    const double covAE = S[4] / dn - (S[2] / dn) * (S[0] / dn);
-    const double covM2E = S[7] / dn - meanM2 * (S[0] / dn);
-    // the bin means' spread, and leave-one-bin-out (jackknife) estimates
-    const double nb = (double)n_bins;
-    double Tot[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    double mbe = 0.0, mba = 0.0;
-    for (int k = 0; k < n_bins; ++k) {
-        for (int q = 0; q < 8; ++q) Tot[q] += s_bin[k][q];
-        mbe += s_bin[k][0] / (double)b;
-        mba += s_bin[k][2] / (double)b;
+    estimates(S, dn, N, T, est);
+    // bin means (their sums divided by the bins) and jackknife estimates of this lane's bins
+    const double mbe = Tot[0] / db / nb, mba = Tot[2] / db / nb, nj = (double)((a.n_bins - 1) * (a.n / a.n_bins));
+    double ve = 0.0, va = 0.0, jk[2][3], jm[3] = {0.0, 0.0, 0.0}, jv[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h;
+        if (k >= a.n_bins) continue;
+        const double xe = bins[k * 8] / db - mbe, xa = bins[k * 8 + 2] / db - mba;
+        ve += xe * xe;
+        va += xa * xa;
+        double R[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) R[q] = Tot[q] - bins[k * 8 + q];
+        estimates(R, nj, N, T, jk[h]);  // shift-invariant forms: the sample's own means enter
+#pragma unroll
+        for (int q = 0; q < 3; ++q) jm[q] += jk[h][q];
     }
-    mbe /= nb;
-    mba /= nb;
-    double vbe = 0.0, vba = 0.0;
-    for (int k = 0; k < n_bins; ++k) {
-        const double de = s_bin[k][0] / (double)b - mbe, da = s_bin[k][2] / (double)b - mba;
-        vbe += de * de;
-        vba += da * da;
-    }
-    const double e_err = sqrt(vbe / (nb - 1.0)) / sqrt(nb) / N;
-    const double m_err = sqrt(vba / (nb - 1.0)) / sqrt(nb) / N;
-    double jm[3] = {0.0, 0.0, 0.0}, jv[3] = {0.0, 0.0, 0.0};
-    const double nj = (double)((n_bins - 1) * b);
-    for (int pass = 0; pass < 2; ++pass)  // mean of the jackknife estimates, then their spread
-        for (int k = 0; k < n_bins; ++k) {
-            double R[8], jk[3];
-            for (int q = 0; q < 8; ++q) R[q] = Tot[q] - s_bin[k][q];
-            estimates(R, nj, N, Tt, jk);  // shift-invariant forms: the sample's own means enter
-            for (int q = 0; q < 3; ++q) {
-                if (pass == 0)
-                    jm[q] += jk[q] / nb;
-                else
-                    jv[q] += (jk[q] - jm[q]) * (jk[q] - jm[q]);
-            }
-        }
-    double *o = out + sid * VEGAS_AVG_FIELDS;
+    ve = warp_sum(ve);
+    va = warp_sum(va);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) jm[q] = warp_sum(jm[q]) / nb;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (lane + 32 * h < a.n_bins)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) jv[q] += (jk[h][q] - jm[q]) * (jk[h][q] - jm[q]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) jv[q] = warp_sum(jv[q]);
+    if (lane != 0) return;
+    double *o = a.out + sid * VEGAS_AVG_FIELDS;
+    const double jf = (nb - 1.0) / nb;
     o[0] = meanE / N;
-    o[1] = e_err;
+    o[1] = sqrt(ve / (nb - 1.0)) / sqrt(nb) / N;
     o[2] = meanA / N;
-    o[3] = m_err;
-    o[4] = est[0];
-    o[5] = sqrt((nb - 1.0) / nb * jv[0]);
-    o[6] = est[1];
-    o[7] = sqrt((nb - 1.0) / nb * jv[1]);
-    o[8] = est[2];
-    o[9] = sqrt((nb - 1.0) / nb * jv[2]);
-    o[10] = -covAE / meanA;
-    o[11] = -covM2E / meanM2;
-    o[12] = tau_e;
-    o[13] = tau_m;
+    o[3] = sqrt(va / (nb - 1.0)) / sqrt(nb) / N;
+    for (int q = 0; q < 3; ++q) {
+        o[4 + 2 * q] = est[q];
+        o[5 + 2 * q] = sqrt(jf * jv[q]);
+    }
+    o[10] = -(S[4] / dn - da * de) / meanA;
+    o[11] = -(S[7] / dn - meanM2 * de) / meanM2;
     o[14] = dn;
     o[15] = nb;
+}
+
+constexpr int kLags = 16;  // lags per pass over the series
+
+// Integrated autocorrelation time of E or |M|, Sokal's window (c = 6): a cluster of blocks per (series,
+// quantity) takes kLags lags at a time (one multiply-add per record and lag, which bounds it; the
+// centred series stays in L1), every block adds the cluster's sums in rank order, and all of them find
+// the same window.
+__global__ void __launch_bounds__(kAnaThreads) thermal_tau_kernel(const ThermalArgs a) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double sm[kLags][kAnaThreads], s_blk[2][kLags];
+    __shared__ double s_tau;
+    __shared__ int s_done;
+    const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank(), lane = threadIdx.x & 31;
+    const int64_t idx = blockIdx.x / CS, which = idx & 1, sid = idx >> 1, n = a.n;
+    const double *x = a.x + (which * a.n_series + sid) * a.stride;
+    const int64_t per = (n + CS - 1) / CS, i0 = rank * per, i1 = min(n, i0 + per);
+    double v[kLags];
+    auto total = [&](int buf) {  // lane q of a warp: the cluster's sum q, in rank order
+        double t = 0.0;
+        if (lane < kLags)
+            for (int b = 0; b < CS; ++b) t += cl.map_shared_rank(&s_blk[buf][0], b)[lane];
+        return t;
+    };
+#pragma unroll
+    for (int q = 0; q < kLags; ++q) v[q] = 0.0;
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kAnaThreads) v[0] += x[i] * x[i];
+    block_sums<kLags>(v, sm, s_blk[0]);
+    if (threadIdx.x == 0) {
+        s_tau = 0.5;
+        s_done = 0;
+    }
+    cl.sync();
+    const double c0 = __shfl_sync(0xFFFFFFFFu, total(0), 0) / (double)n;
+    int buf = 1;
+    for (int64_t t0 = 1; t0 <= n / 2 && c0 != 0.0; t0 += kLags, buf ^= 1) {
+#pragma unroll
+        for (int q = 0; q < kLags; ++q) v[q] = 0.0;
+        const int64_t e = min(i1, n - t0);
+        for (int64_t i = i0 + threadIdx.x; i < e; i += kAnaThreads) {
+            const double xi = x[i];
+            const double *y = x + i + t0;  // zeros from n on
+#pragma unroll
+            for (int q = 0; q < kLags; ++q) v[q] = fma(xi, y[q], v[q]);
+        }
+        block_sums<kLags>(v, sm, s_blk[buf]);
+        cl.sync();  // every block's sums are there (and nobody reads the other buffer any more)
+        if (threadIdx.x < 32) {
+            const int64_t t = t0 + lane;
+            const bool in = lane < kLags && t <= n / 2;
+            const double rho = in ? total(buf) / (double)(n - t) / c0 : 0.0;
+            double run = s_tau, mine = run;  // partial sums in lag order
+            for (int q = 0; q < kLags; ++q) {
+                run += __shfl_sync(0xFFFFFFFFu, rho, q);
+                if (lane == q) mine = run;
+            }
+            const uint32_t closed = __ballot_sync(0xFFFFFFFFu, in && (double)t >= 6.0 * mine);
+            const double end = __shfl_sync(0xFFFFFFFFu, mine, closed ? __ffs(closed) - 1 : kLags - 1);
+            if (lane == 0) {
+                s_tau = end;
+                s_done = closed != 0u;
+            }
+        }
+        __syncthreads();
+        if (s_done) break;
+    }
+    if (rank == 0 && threadIdx.x == 0) a.out[sid * VEGAS_AVG_FIELDS + 12 + which] = s_tau;
+    cl.sync();  // no block leaves while another may read its sums
 }
 
 // ------------------------------------------------------------------ reweighting
@@ -474,16 +588,66 @@ extern "C" vegas_status vegas_thermal_averages(const double *series, int64_t n_s
         vegas_status st = have_device();
         if (st != VEGAS_OK) return st;
         cudaStream_t stream = (cudaStream_t)cuda_stream;
-        const size_t hb = sizeof(double) * 4 * (size_t)n_series * (size_t)len;
-        const size_t sb = sizeof(double) * (size_t)n_series, ob = VEGAS_AVG_FIELDS * sb;
+        int dev = 0, sms = 1;
+        ACK(cudaGetDevice(&dev));
+        ACK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        ThermalArgs a{};
+        a.len = len;
+        a.cut = cut;
+        a.n = len - cut;
+        a.n_series = (int32_t)n_series;
+        a.n_bins = n_bins;
+        a.stride = a.n + kLags;
+        a.chunk = std::max<int64_t>(1024, (a.n + 63) / 64);
+        a.chunks = (int32_t)((a.n + a.chunk - 1) / a.chunk);
+        const size_t D = sizeof(double), ns = (size_t)n_series, hb = D * 4 * ns * (size_t)len, sb = D * ns;
+        const size_t xb = D * 2 * ns * (size_t)a.stride, cb = D * 2 * ns * (size_t)a.chunks, bb = D * 8 * ns * (size_t)(n_bins + 1);
+        const size_t ob = VEGAS_AVG_FIELDS * sb;
         DevBuf b;
-        for (const size_t x : {hb, sb, sb, ob}) b.reserve(x);
+        for (const size_t x : {hb, xb, cb, bb, sb, sb, ob}) b.reserve(x);
         ACK(b.allocate());
-        double *d_h = b.take<double>(hb), *d_T = b.take<double>(sb), *d_N = b.take<double>(sb), *d_out = b.take<double>(ob);
+        double *d_h = b.take<double>(hb);
+        a.series = d_h;
+        a.x = b.take<double>(xb);
+        a.sums = b.take<double>(cb);
+        a.bins = b.take<double>(bb);
+        double *d_T = b.take<double>(sb), *d_N = b.take<double>(sb), *d_out = b.take<double>(ob);
+        a.T = d_T;
+        a.Nsites = d_N;
+        a.out = d_out;
         ACK(cudaMemcpyAsync(d_h, series, hb, cudaMemcpyHostToDevice, stream));
         ACK(cudaMemcpyAsync(d_T, T, sizeof(double) * n_series, cudaMemcpyHostToDevice, stream));
         ACK(cudaMemcpyAsync(d_N, n_sites, sizeof(double) * n_series, cudaMemcpyHostToDevice, stream));
-        thermal_kernel<<<(unsigned)n_series, kAnaThreads, 0, stream>>>(d_h, len, cut, n_bins, d_T, d_N, d_out);
+        // series per launch: a grid's second dimension holds at most 65535
+        for (int64_t s0 = 0; s0 < n_series; s0 += 65535) {
+            ThermalArgs p = a;
+            const unsigned m = (unsigned)std::min<int64_t>(65535, n_series - s0);
+            p.n_series = (int32_t)n_series;  // rows of x between E and |M|
+            p.series += s0 * len * 4;
+            p.x += s0 * a.stride;
+            p.sums += s0 * a.chunks * 2;
+            p.bins += s0 * (n_bins + 1) * 8;
+            p.T += s0;
+            p.Nsites += s0;
+            p.out += s0 * VEGAS_AVG_FIELDS;
+            thermal_load_kernel<<<dim3((unsigned)a.chunks, m), kAnaThreads, 0, stream>>>(p);
+            thermal_bin_kernel<<<dim3((unsigned)n_bins + 1u, m), kAnaThreads, 0, stream>>>(p);
+            thermal_estimate_kernel<<<m, 32, 0, stream>>>(p);
+            int cs = 1;  // blocks per cluster: as many as keep one block per SM, at most 8
+            while (cs < 8 && (int64_t)m * 2 * (cs * 2) <= sms) cs *= 2;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(m * 2u * (unsigned)cs);
+            cfg.blockDim = dim3(kAnaThreads);
+            cfg.stream = stream;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)cs;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            ACK(cudaLaunchKernelEx(&cfg, thermal_tau_kernel, p));
+        }
         ACK(cudaGetLastError());
         ACK(cudaMemcpyAsync(out, d_out, sizeof(double) * VEGAS_AVG_FIELDS * n_series, cudaMemcpyDeviceToHost, stream));
         ACK(cudaStreamSynchronize(stream));

@@ -1,0 +1,51 @@
+"""Thermal averages over the kernels' dispatch (chunks, bins and records behind them, lags per pass,
+blocks per cluster) against the numpy oracle in FP64."""
+
+import numpy as np
+import pytest
+
+from oracle import analysis
+import paper_1803_07030_gb300 as vg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    vg.build()
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+@pytest.mark.parametrize("ns, length, cut, bins, tau", [
+    (1, 2, 0, 2, 1.0),            # one record per bin, one lag
+    (1, 40, 3, 7, 1.0),           # records behind the bins
+    (3, 131, 100, 31, 2.0),
+    (2, 1025, 1, 64, 3.0),        # two chunks of the load, most bins
+    (1, 30000, 0, 20, 100.0),     # many lag passes, clusters of eight
+    (20, 3000, 10, 33, 5.0),
+    (77, 500, 100, 20, 4.0),      # no clusters
+    (200, 333, 3, 10, 2.0),
+])
+def test_averages_match_oracle(ns, length, cut, bins, tau):
+    rng = np.random.default_rng(ns + length)
+    a = np.exp(-1.0 / tau)
+    x = rng.normal(size=(length, ns, 4))
+    for i in range(1, length):
+        x[i] = a * x[i - 1] + np.sqrt(1 - a * a) * x[i]
+    H = np.ascontiguousarray(np.swapaxes(x, 0, 1)) * np.array([20.0, 30.0, 30.0, 30.0]) + np.array([-3000.0, 0.0, 0.0, 200.0])
+    T = np.linspace(0.5, 2.0, ns)
+    out = vg.thermal_averages(H, cut, bins, T, 1000.0)
+    for s in range(ns):
+        ref = analysis.thermal_averages(H[s], cut, bins, T[s], 1000.0)
+        for k, name in enumerate(vg.AVG_FIELDS):
+            # sums of up to 30,000 centred terms in FP64, and differences of quantities 1e2 larger
+            assert abs(out[s, k] - ref[name]) <= 1e-9 * abs(ref[name]) + 1e-9 * (3000.0 if name in ("v1", "v2") else 1e-3), (
+                s, name, out[s, k], ref[name])
+
+
+def test_constant_series_has_no_correlation_time():
+    H = np.tile(np.array([-5.0, 0.0, 3.0, 4.0]), (2, 100, 1))
+    out = vg.thermal_averages(H, 10, 5, 1.0, 10.0)
+    assert np.allclose(out[:, [12, 13]], 0.5) and np.allclose(out[:, 0], -0.5) and np.allclose(out[:, 2], 0.5)
