@@ -133,6 +133,7 @@ struct vegas_ctx {
     bool tile_ok = false;
     bool use_tile = false;  // the cooperative sweep runs it (not while the autotuner times the sweeps)
     TileArgs tile{};
+    Tile64Args tile64{};  // its FP64 counterpart (uniform trials)
     int tile_threads = 0;
     size_t tile_smem_bytes = 0;
     std::vector<void *> tile_bufs;
@@ -368,11 +369,20 @@ int64_t coop_kernels(const vegas_ctx *c, int32_t n) {
 // one that writes their records); the run state advances afterwards.
 void enqueue_coop(vegas_ctx *c, cudaStream_t st, int32_t n) {
     if (c->use_tile) {
-        TileArgs a = c->tile;
         for (int32_t m = 0; m < n; m += kTileMcs) {
-            a.mcs = std::min(kTileMcs, n - m);
-            if (launch_tile(a, c->tile_threads, c->tile_smem_bytes, st) != 0) return;
-            launch_advance(c->d_run, a.mcs, st);
+            const int32_t k = std::min(kTileMcs, n - m);
+            int e;
+            if (c->precision == 64) {
+                Tile64Args a = c->tile64;
+                a.t.mcs = k;
+                e = launch_tile64(a, c->tile_threads, c->tile_smem_bytes, st);
+            } else {
+                TileArgs a = c->tile;
+                a.mcs = k;
+                e = launch_tile(a, c->tile_threads, c->tile_smem_bytes, st);
+            }
+            if (e != 0) return;
+            launch_advance(c->d_run, k, st);
         }
         return;
     }
@@ -572,9 +582,10 @@ bool class1_block_deps(const SampleInfo &si, const LoadedSample &l, int bs, int 
     return true;
 }
 
-// The tiled form of the cooperative sweep for the context's one FP32 sample: parts of at least
-// kTilePerClass sites of the widest class, at most one block per SM over all replicas. Leaves
-// tile_ok unset when its rows are longer than kEllRow or a part does not fit in shared memory.
+// The tiled form of the cooperative sweep for the context's one sample: parts of at least
+// kTilePerClass (FP64: kTile64PerClass) sites of the widest class, at most one block per SM over
+// all replicas. Leaves tile_ok unset when its rows are longer than kEllRow, a part does not fit in
+// shared memory, or (FP64) the sample has update policies.
 vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     const SampleInfo &si = c->samples[0];
     const vegas_options &o = c->opt;
@@ -587,7 +598,10 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     TileShape ts{};
     ts.n = si.n;
     ts.n_colours = si.n_colours;
-    ts.parts = std::min(blocks / c->R, (widest + kTilePerClass - 1) / kTilePerClass);
+    const bool p64 = c->precision == 64;
+    if (p64 && si.has_policy) return VEGAS_OK;
+    const int per = p64 ? kTile64PerClass : kTilePerClass;
+    ts.parts = std::min(blocks / c->R, (widest + per - 1) / per);
     ts.width = si.uniform_degree == 6 ? 6 : kEllRow;
     ts.site_off = si.site_off;
     ts.cstart = l.cstart.data();
@@ -614,7 +628,15 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
         a.rk0[q] = (uint32_t)o.seed + q * 0x9E3779B9u;
         a.rk1[q] = (uint32_t)(o.seed >> 32) + q * 0xBB67AE85u;
     }
-    c->tile_threads = tile_shape(a, ts, plan, &c->tile_smem_bytes);
+    std::vector<double> J64;
+    if (p64) {
+        c->tile64 = Tile64Args{};
+        c->tile64.t = a;
+        c->tile_threads = tile64_shape(c->tile64, ts, plan, J64, &c->tile_smem_bytes);
+        a = c->tile64.t;
+    } else {
+        c->tile_threads = tile_shape(a, ts, plan, &c->tile_smem_bytes);
+    }
     cudaGetLastError();
     if (c->tile_threads == 0) return VEGAS_OK;
     auto up = [&](auto *&p, const void *src, size_t bytes) {
@@ -634,11 +656,13 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     CK(c, up(a.pub, plan.pub.data(), plan.pub.size() * sizeof(int32_t)));
     CK(c, up(a.rows, plan.rows.get(), plan.row_bytes));
     CK(c, up(a.codes, plan.codes.data(), plan.codes.size() * sizeof(float)));
-    CK(c, up(a.mail, nullptr, (size_t)plan.n_mail * c->R * sizeof(float4)));
+    CK(c, up(a.mail, nullptr, (size_t)plan.n_mail * c->R * sizeof(float4) * (p64 ? 2 : 1)));
+    if (p64) CK(c, up(c->tile64.J, J64.data(), J64.size() * sizeof(double)));
     CK(c, up(a.partial, nullptr, words * 4 * sizeof(double)));
     CK(c, up(a.count, nullptr, words * sizeof(uint32_t)));
     CK(c, up(a.abort, nullptr, sizeof(uint32_t)));
     CK(c, cudaStreamSynchronize(c->stream));  // the plan goes out of scope
+    c->tile64.t = a;
     c->tile_ok = true;
     return VEGAS_OK;
 }
@@ -1294,7 +1318,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         // (the resident sweep's, or built here), read without row offsets
         const int deg0 = c->passes[0].args.deg;
         bool use_ell = false;
-        if (!p64) TRY(make_tile(c, L[0]));
+        TRY(make_tile(c, L[0]));
         if (!p64 && deg0 != 6) {
             int64_t max_deg = 0;
             for (int64_t g = 0; g < n_sites; ++g)
@@ -1512,6 +1536,12 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         c->tuned = true;
     } else if (o.variant == 0 || (!c->res_eligible && !c->coop_eligible && !c->cluster_eligible)) {
         c->variant = 0;
+        c->tuned = true;
+    } else if (p64 && c->tile_ok) {
+        // FP64, and the tiled form fits: several times faster than the others (8^3: 4.4 us per MCS
+        // against 24), and every sweep records the same FP64 sums to their rounding
+        c->variant = 2;
+        c->use_tile = true;
         c->tuned = true;
     } else {
         // automatic: timed on the first run; until then, the shape suggests one
@@ -2258,7 +2288,8 @@ extern "C" vegas_status vegas_stats(const vegas_ctx *c, vegas_stats_t *o) {
         o->n_types = c->n_types;
         o->snapshot_steps = c->snapshot_steps;
         o->block_threads = c->variant == 1 ? c->res_threads : (c->variant == 3 ? c->cluster_threads : kThreads);
-        if (c->variant == 2 && c->use_tile) o->block_threads = c->tile_threads + kTileRecord;
+        if (c->variant == 2 && c->use_tile)
+            o->block_threads = c->tile_threads + (c->precision == 64 ? kTile64Trial + 32 : kTileRecord);
         o->cluster_blocks = c->variant == 3 ? c->cluster_cs : 0;
         o->split_sites = c->variant == 3 ? c->res.split_sites : 0;
         o->group_threads = (c->variant == 1 || c->variant == 3) ? c->res.group_threads : 0;

@@ -24,41 +24,11 @@
 #include <cstdint>
 
 #include "vegas_device.cuh"
+#include "vegas_fp64.cuh"
 #include "vegas_internal.h"
 
 namespace vegas {
 namespace {
-
-// ------------------------------------------------------------------ FP64 helpers
-// Explicit round-to-nearest operations: the compiler may not fuse them, which keeps the
-// FP64 path identical to the CPU oracle built without contraction.
-__device__ __forceinline__ double dm(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double da(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double ds(double a, double b) { return __dsub_rn(a, b); }
-
-// Uniform in [0, 1) with 53 bits: (hi * 2^21 + (lo >> 11)) * 2^-53 (exact).
-__device__ __forceinline__ double u53(uint32_t hi, uint32_t lo) {
-    const unsigned long long m = ((unsigned long long)hi << 21) | (unsigned long long)(lo >> 11);
-    return __dmul_rn(__ull2double_rn(m), 0x1p-53);
-}
-
-// Point on the unit sphere by Marsaglia's method (Ann. Math. Stat. 43, 1972): draw
-// (u1, u2) uniform in the square [-1, 1)^2 until s = u1^2 + u2^2 < 1, then
-// (2 u1 sqrt(1-s), 2 u2 sqrt(1-s), 1 - 2 s). Candidate k uses counter word 3 = purpose|k.
-__device__ double3 sphere64(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t purpose, uint32_t k0, uint32_t k1,
-                            uint32_t *err) {
-    for (uint32_t k = 0; k < 64; ++k) {
-        const uint4 w = philox10(make_uint4(c0, c1, c2, purpose | k), k0, k1);
-        const double u1 = ds(dm(2.0, u53(w.x, w.y)), 1.0);
-        const double u2 = ds(dm(2.0, u53(w.z, w.w)), 1.0);
-        const double s = da(dm(u1, u1), dm(u2, u2));
-        if (s >= 1.0) continue;
-        const double q = __dsqrt_rn(ds(1.0, s));
-        return make_double3(dm(dm(2.0, u1), q), dm(dm(2.0, u2), q), ds(1.0, dm(2.0, s)));
-    }
-    atomicOr(err, kErrSphere);
-    return make_double3(0.0, 0.0, 1.0);
-}
 
 __device__ __forceinline__ double cub64(double x, double y, double z) {
     const double xx = dm(x, x), yy = dm(y, y), zz = dm(z, z);
@@ -268,12 +238,11 @@ __device__ __forceinline__ void site64(const PassArgs &a, int g, int r, int R, u
         dE = da(da(dEex, dEan), dEcub);
     }
     // Metropolis acceptance (Eq. 4), k_B = 1
-    bool acc;
-    if (dE <= 0.0) {
-        acc = true;
-    } else {
+    bool acc = true;
+    if (dE > 0.0) {
         const uint4 wa = philox10(make_uint4(orig, t, inst, kPurposeAccept64), k0, k1);
-        acc = u53(wa.x, wa.y) < exp(-dm(beta, dE));
+        acc = accept64(__double_as_longlong(dE), dE, beta, (float)beta,
+                       ((unsigned long long)wa.x << 21) | (unsigned long long)(wa.y >> 11));
     }
     if (isnan(dE)) {
         atomicOr(a.err, kErrNaN);

@@ -42,6 +42,7 @@
 
 #include "vegas_device.cuh"
 #include "vegas_internal.h"
+#include "vegas_tile.cuh"
 #include "vegas_tile.h"
 
 namespace vegas {
@@ -50,45 +51,6 @@ namespace {
 // Named barriers: the sweeping threads among themselves; the two partial-sum buffers between
 // them and the record warp (full: the sums are written, empty: the record warp has read them).
 constexpr int kBarSweep = 1, kBarFull = 2, kBarEmpty = 4;
-
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
-// A mailbox word in one 128-bit access (single-copy atomic), through L2.
-__device__ __forceinline__ void mail_store(float4 *p, float x, float y, float z, uint32_t tag) {
-    const uint64_t lo = (uint64_t)__float_as_uint(x) | (uint64_t)__float_as_uint(y) << 32;
-    const uint64_t hi = (uint64_t)__float_as_uint(z) | (uint64_t)tag << 32;
-    asm volatile("{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(p), "l"(lo),
-                 "l"(hi)
-                 : "memory");
-}
-__device__ __forceinline__ float4 mail_load(const float4 *p) {
-    uint64_t lo, hi;
-    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
-                 : "=l"(lo), "=l"(hi)
-                 : "l"(p)
-                 : "memory");
-    return make_float4(__uint_as_float((uint32_t)lo), __uint_as_float((uint32_t)(lo >> 32)), __uint_as_float((uint32_t)hi),
-                       __uint_as_float((uint32_t)(hi >> 32)));
-}
-
-// The barrier and the logical and of every thread's ok.
-__device__ __forceinline__ bool bar_and(int id, int n, bool ok) {
-    int all;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.and.pred q, %2, %3, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
-                 : "=r"(all)
-                 : "r"((int)ok), "r"(id), "r"(n)
-                 : "memory");
-    return all != 0;
-}
-
-__device__ __forceinline__ uint64_t tile_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 
 // The spin of local site i: x and y as one 8-byte pair, z in an array of its own (two loads).
 __device__ __forceinline__ float4 loc_spin(const float *sp, int cap, int i) {
@@ -643,6 +605,8 @@ size_t tile_layout(TileArgs &a, const TilePlan &p, int threads) {
 
 }  // namespace
 
+void tile_tables(const TileArgs &a, const TileShape &s, TilePlan &p) { write_tables(a, s, p); }
+
 // Raises the kernel's shared-memory limit to the device's (not to this plan's size: the limit
 // belongs to the kernel, which other contexts launch too).
 int tile_shape(TileArgs &a, const TileShape &s, TilePlan &p, size_t *smem) {
@@ -717,8 +681,12 @@ int launch_tile(const TileArgs &a, int threads, size_t smem, void *stream) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if ((e = cudaLaunchKernelEx(&cfg, select_tile(a), a)) != cudaSuccess) return (int)e;
+    return launch_tile_record(a, stream);
+}
+
+int launch_tile_record(const TileArgs &a, void *stream) {
     const int64_t warps = (int64_t)a.mcs << a.pass.log2R;
-    tile_record_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(a);
+    tile_record_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, (cudaStream_t)stream>>>(a);
     return (int)cudaGetLastError();
 }
 

@@ -80,6 +80,31 @@ bool tile_plan(const TileShape &s, TilePlan &out);
 // Chooses the threads per block and what it keeps in shared memory, and writes the rows; 0 when
 // the parts do not fit.
 int tile_shape(TileArgs &a, const TileShape &s, TilePlan &p, size_t *smem);
+void tile_tables(const TileArgs &a, const TileShape &s, TilePlan &p);  // the host side of those tables
+int launch_tile_record(const TileArgs &a, void *stream);  // the records of a launch's MCS
+
+// ---- FP64 (vegas_tile64.cu)
+constexpr int kTile64Threads = 256;   // most sweeping threads per block
+constexpr int kTile64Trial = 64;      // threads that draw trials
+constexpr int kTile64Ahead = 4;       // classes of trials drawn ahead
+constexpr int kTile64PerClass = 10;   // sites of the widest class per part
+constexpr int kTile64Sites = 96;      // most sites of a class in a part
+
+struct Tile64Trial {
+    double x, y, z;        // trial spin
+    unsigned long long u;  // acceptance uniform, u 2^-53
+};
+
+struct Tile64Args {
+    TileArgs t;            // rows: words (local site | lower flag << 16); mail: two words per site
+    const double *J;       // [own site][width]
+    int32_t J_off, trial_off, widest;
+};
+
+// Threads that sweep, and the tables (J beside the plan's rows); 0 when the parts do not fit.
+int tile64_shape(Tile64Args &a, const TileShape &s, TilePlan &p, std::vector<double> &J, size_t *smem);
+int launch_tile64(const Tile64Args &a, int threads, size_t smem, void *stream);
+
 // Sweep of a.mcs MCS and their records; returns the CUDA error.
 int launch_tile(const TileArgs &a, int threads, size_t smem, void *stream);
 

@@ -113,3 +113,52 @@ def test_automatic_choice_keeps_the_chain(make, R):
         for i in {0, R - 1}:
             assert np.array_equal(a.spins(i), b.spins(i))
         assert np.array_equal(a.accept_history(), b.accept_history())
+
+
+FP64 = {
+    "one_site": (lambda: free_spins(1, field_axis=(0, 0, 1)), 1, {}),
+    "sc6_anisotropic": (lambda: sc_periodic(6, k_uni=0.3, e_axis=(1, 1, 0)), 2, {}),
+    "odd_sides": (lambda: sc_periodic((5, 7, 9), bimodal_seed=1), 1, {}),
+    "all_terms": (lambda: _sparse(8), 4, {}),
+    "several_rounds": (lambda: sc_periodic(8, bimodal_seed=3), 32, {}),       # 64 sites of a class per part
+    "two_blocks": (lambda: sc_periodic((4, 4, 6)), 1, {"max_blocks": 2}),
+    "fcc": (lambda: fcc_sphere(4.2), 3 + 1, {}),
+    "core_shell": (lambda: core_shell_particle(4, radius=5.0, core_radius=3.5), 1, {}),
+}
+
+
+@pytest.mark.parametrize("name", list(FP64))
+def test_fp64_tiled_sweep_equals_oracle(name):
+    import oracle
+
+    make, R, kw = FP64[name]
+    s = make()
+    mcs = 6
+    T = np.stack([[2.0 - 0.02 * r, 0.02, 0.6] for r in range(R)])  # a cold step: decisions far out in the tail
+    B = np.stack([[0.3, -0.2, 0.1 * r] for r in range(R)])
+    with vg.Context([s], precision=64, replicas=R, seed=9, variant=2, accept_log_mcs=3 * mcs, stream=None, **kw) as c:
+        c.run(T, B, mcs)
+        assert c.stats()["block_threads"] % 32 == 0 and c.stats()["block_threads"] > 32  # the tiled form
+        ref = oracle.run(s, T, B, mcs, seed=9, log_mcs=3 * mcs, n_threads=R)
+        assert ref["err"] == 0
+        alog = c.accept_log().reshape(3 * mcs, R, -1)
+        for r in range(R):
+            assert np.array_equal(c.spins(r), ref["spins"][r]), r
+            assert np.array_equal(alog[:, r], ref["accept_log"][r]), r
+            assert np.array_equal(c.accept_history()[r], ref["accepted"][r]), r
+            assert np.allclose(c.history()[r], ref["history"][r], rtol=1e-12, atol=1e-12 * s.n_sites * 8)
+
+
+def test_fp64_long_step_and_counter_set_back():
+    s = sc_periodic(6)
+    T = np.array([[0.9], [1.3]])
+    with vg.Context([s], precision=64, replicas=2, seed=7, variant=0, stream=None) as a, \
+            vg.Context([s], precision=64, replicas=2, seed=7, stream=None) as b:
+        for c in (a, b):
+            c.run(T, 0 * T, 1100)
+            c.set_mcs_counter(3)
+            c.run(T, 0 * T, 40)
+        for i in range(2):
+            assert np.array_equal(a.spins(i), b.spins(i))
+        assert np.array_equal(a.accept_history(), b.accept_history())
+        assert np.allclose(a.history(), b.history(), rtol=1e-12, atol=1e-10)
