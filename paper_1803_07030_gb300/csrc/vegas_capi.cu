@@ -77,6 +77,9 @@ struct vegas_ctx {
     // device buffers
     void *d_spins = nullptr, *d_edges = nullptr, *d_p0 = nullptr, *d_p1 = nullptr, *d_pk = nullptr;
     int2 *d_ell = nullptr;  // links as fixed rows of kEllRow (spins-in-shared-memory sweeps)
+    void *d_batch_rows = nullptr;  // rows, exchange values and lower modes of batch32_kernel
+    float *d_batch_codes = nullptr;
+    int32_t *d_batch_modes = nullptr;
     int64_t *d_rowptr = nullptr, *d_slot_base = nullptr;
     uint32_t *d_pass_tickets = nullptr;  // [passes] block counters of the R = 32 staged kernel
     int32_t n_groups = 1;      // type groups of the partial slots (n_types with type_stats)
@@ -112,6 +115,8 @@ struct vegas_ctx {
     bool res_smem_eligible = false;  // every instance's spins fit the shared-memory form
     bool res_smem = false;           // the resident sweep keeps spins in shared memory
     bool cluster_smem = false;       // the cluster sweep keeps copies of the spins in shared memory
+    bool batch_ok = false;           // both run as batch32_kernel (uniform trials, no per-type sums)
+    BatchArgs batch{};               // its tables
     int res_items = 0;          // instances of the resident and cluster sweeps
     bool res_policy = false;    // some sample has a policy table (kernel choice for the shapes)
     bool res_eligible = false, tuned = false;
@@ -220,7 +225,7 @@ void free_all(vegas_ctx *c) {
     for (cudaGraph_t g : c->run_graph_defs) cudaGraphDestroy(g);
     if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
     if (c->graph) cudaGraphDestroy(c->graph);
-    void *bufs[] = {c->d_spins, c->d_edges, c->d_ell, c->d_p0, c->d_p1, c->d_pk, c->d_rowptr, c->d_slot_base, c->d_orig,
+    void *bufs[] = {c->d_spins, c->d_edges, c->d_ell, c->d_batch_rows, c->d_batch_codes, c->d_batch_modes, c->d_p0, c->d_p1, c->d_pk, c->d_rowptr, c->d_slot_base, c->d_orig,
                     c->d_slot_count, c->d_norm, c->d_partial, c->d_sched, c->d_hist, c->d_run, c->d_err, c->d_alog,
                     c->d_insts, c->d_cstart, c->d_queue, c->d_bar, c->d_coop_partial, c->d_acc, c->d_acc_hist,
                     c->d_pol, c->d_pol32, c->d_qis, c->d_sigma, c->d_adapt_n, c->d_type_hist, c->d_snap, c->d_segs,
@@ -257,6 +262,11 @@ int ilog2(int v) {
 // the spins in global memory, when that form does not fit the device.
 constexpr int64_t kResSmemBytes = 200 * 1024;  // spins in shared memory: 12 bytes per site
 
+// The shared-memory forms run as batch32_kernel (blocks of 512 threads, groups of at least 128).
+bool batch_form(const vegas_ctx *c, int threads, int group_threads) {
+    return c->batch_ok && threads == kBatchThreads && (group_threads == 0 || group_threads >= 128);
+}
+
 bool set_resident_shape(vegas_ctx *c, int threads, int group_threads = 0, int group_sites = 0, bool smem = false) {
     const bool grouped = group_threads > 0 && group_threads < threads && threads % group_threads == 0 &&
                          threads / group_threads <= 15;
@@ -268,7 +278,10 @@ bool set_resident_shape(vegas_ctx *c, int threads, int group_threads = 0, int gr
         if (grouped)  // an even cap: the groups' regions then keep the budget with even starts
             a.group_sites = (int)std::min<int64_t>(group_sites, (kResSmemBytes / (12 * (threads / group_threads))) & ~1);
         a.smem_sites = c->max_instance_sites;
-        const int bps = resident_blocks_per_sm(threads, c->res_policy, resident_smem_bytes(a, threads));
+        BatchArgs ba = c->batch;
+        ba.r = a;
+        const int bps = batch_form(c, threads, a.group_threads) ? batch_capacity(ba, 1, 1)
+                                    : resident_blocks_per_sm(threads, c->res_policy, resident_smem_bytes(a, threads));
         cudaGetLastError();
         if (bps > 0) {
             c->res.group_sites = a.group_sites;
@@ -301,7 +314,11 @@ bool set_cluster_shape(vegas_ctx *c, int cs, int threads, int split = 0, int gro
     if (smem && a.group_threads > 0)
         a.group_sites = (int)std::min<int64_t>(a.group_sites, (kResSmemBytes / (12 * (threads / a.group_threads))) & ~1);
     a.smem_sites = smem ? c->max_instance_sites : 0;
-    const int cap = cluster_capacity(cs, threads, c->res_policy, cluster_smem_bytes(a, threads));
+    BatchArgs ba = c->batch;
+    ba.r = a;
+    const int cap = smem && batch_form(c, threads, a.group_threads)
+                        ? batch_capacity(ba, cs, c->sm_count)
+                        : cluster_capacity(cs, threads, c->res_policy, cluster_smem_bytes(a, threads));
     cudaGetLastError();
     if (cap <= 0) return false;
     c->cluster_cs = cs;
@@ -356,7 +373,13 @@ void enqueue_resident(vegas_ctx *c, cudaStream_t st, int32_t n) {
     ResidentArgs a = c->res;
     a.mcs = n;
     a.smem_sites = c->res_smem ? c->max_instance_sites : 0;
-    launch_resident(a, c->res_grid, c->res_threads, st);
+    if (c->res_smem && batch_form(c, c->res_threads, a.group_threads)) {
+        BatchArgs ba = c->batch;
+        ba.r = a;
+        launch_batch(ba, c->res_grid, 1, st);
+    } else {
+        launch_resident(a, c->res_grid, c->res_threads, st);
+    }
     launch_advance(c->d_run, n, st);
 }
 
@@ -399,7 +422,13 @@ void enqueue_cluster(vegas_ctx *c, cudaStream_t st, int32_t n) {
     ResidentArgs a = c->res;
     a.mcs = n;
     a.smem_sites = c->cluster_smem ? c->max_instance_sites : 0;
-    launch_cluster(a, c->cluster_n, c->cluster_cs, c->cluster_threads, st);
+    if (c->cluster_smem && batch_form(c, c->cluster_threads, a.group_threads)) {
+        BatchArgs ba = c->batch;
+        ba.r = a;
+        launch_batch(ba, c->cluster_n, c->cluster_cs, st);
+    } else {
+        launch_cluster(a, c->cluster_n, c->cluster_cs, c->cluster_threads, st);
+    }
     launch_advance(c->d_run, n, st);
 }
 
@@ -1248,8 +1277,72 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         for (int64_t g = 0; g < n_sites; ++g) max_deg = std::max(max_deg, h_rowptr[(size_t)g + 1] - h_rowptr[(size_t)g]);
         c->res_smem_eligible = o.resident_smem >= 0 && 12 * (int64_t)c->max_instance_sites <= kResSmemBytes &&
                                max_deg <= kEllRow;
-        if (c->res_smem_eligible) {
-            std::vector<int2> h_ell((size_t)n_sites * kEllRow, make_int2(-1, 0));
+        c->batch_ok = c->res_smem_eligible && !any_policy && c->n_types == 0;
+        std::vector<int2> h_ell;           // outlive the uploads below
+        std::vector<uint32_t> h_rows;
+        std::vector<float> h_codes;
+        std::vector<int32_t> h_modes;
+        if (c->batch_ok) {
+            // the samples' exchange values, when they are few: rows are then words
+            auto code_of = [&](float v) {
+                size_t k = 0;
+                while (k < h_codes.size() && h_codes[k] != v) ++k;
+                if (k == h_codes.size()) h_codes.push_back(v);
+                return (uint32_t)k;
+            };
+            code_of(0.0f);  // padding
+            for (int32_t s = 0; s < n_samples && h_codes.size() <= (size_t)kTileCodes; ++s)
+                for (const double v : L[(size_t)s].J) {
+                    code_of((float)v);
+                    if (h_codes.size() > (size_t)kTileCodes) break;
+                }
+            const bool words = h_codes.size() <= (size_t)kTileCodes;
+            const int per = words ? 1 : 2;
+            h_rows.resize((size_t)n_sites * kEllRow * per);
+            BatchArgs &ba = c->batch;
+            ba = BatchArgs{};
+            for (int32_t s = 0; s < n_samples; ++s) {
+                const LoadedSample &l = L[(size_t)s];
+                const SampleInfo &si = c->samples[(size_t)s];
+                for (double x : l.k_cub) ba.cubic |= x != 0.0 ? 1 : 0;
+                for (int32_t q = 0; q < l.n_colours; ++q)
+                    for (int32_t g = l.cstart[(size_t)q]; g < l.cstart[(size_t)q + 1]; ++g) {
+                        uint32_t *row = &h_rows[(size_t)(si.site_off + g) * kEllRow * per];
+                        const int64_t e0 = l.row_ptr[(size_t)g], deg = l.row_ptr[(size_t)g + 1] - e0;
+                        for (int w = 0; w < kEllRow; ++w) {
+                            const bool in = w < deg;
+                            const int32_t j = in ? l.col[(size_t)(e0 + w)] : g;
+                            const float J = in ? (float)l.J[(size_t)(e0 + w)] : 0.0f;
+                            const uint32_t link = (uint32_t)j | (in && j < l.cstart[(size_t)q] ? 0x10000u : 0u);
+                            if (words) {
+                                row[w] = link | code_of(J) << 17;
+                            } else {
+                                row[2 * w] = link;
+                                row[2 * w + 1] = (uint32_t)float_bits(J);
+                            }
+                        }
+                    }
+            }
+            for (const PassLaunch &pl : c->passes) h_modes.push_back(pl.args.lower_mode);  // segments are the passes in order
+            ba.cubic = ba.cubic ? 1 : 0;
+            ba.n_codes = words ? (int32_t)h_codes.size() : 0;
+            for (uint32_t q = 0; q < 10; ++q) {
+                ba.rk0[q] = (uint32_t)o.seed + q * 0x9E3779B9u;
+                ba.rk1[q] = (uint32_t)(o.seed >> 32) + q * 0xBB67AE85u;
+            }
+            DALLOC(c->d_batch_rows, sizeof(uint32_t) * h_rows.size());
+            DALLOC(c->d_batch_codes, sizeof(float) * h_codes.size());
+            DALLOC(c->d_batch_modes, sizeof(int32_t) * std::max<size_t>(h_modes.size(), 1));
+            H2D(c->d_batch_rows, h_rows.data(), sizeof(uint32_t) * h_rows.size());
+            H2D(c->d_batch_codes, h_codes.data(), sizeof(float) * h_codes.size());
+            if (!h_modes.empty()) H2D(c->d_batch_modes, h_modes.data(), sizeof(int32_t) * h_modes.size());
+            ba.rows = c->d_batch_rows;
+            ba.codes = c->d_batch_codes;
+            ba.modes = c->d_batch_modes;
+        }
+        // the forms with policies or per-type sums, and blocks of 256 or groups of 64 threads when asked for
+        if (c->res_smem_eligible && (!c->batch_ok || o.group_threads == 64 || o.resident_smem == 1)) {
+            h_ell.assign((size_t)n_sites * kEllRow, make_int2(-1, 0));
             for (int64_t g = 0; g < n_sites; ++g)
                 for (int64_t e = h_rowptr[(size_t)g]; e < h_rowptr[(size_t)g + 1]; ++e)
                     h_ell[(size_t)g * kEllRow + (size_t)(e - h_rowptr[(size_t)g])] = h_e32[(size_t)e];
@@ -1309,6 +1402,10 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
                                                         o.variant == 3 && o.resident_smem == 1);
             }
             cudaGetLastError();  // an unsupported cluster shape only makes the sweep ineligible
+        }
+        if (cudaStreamSynchronize(c->stream) != cudaSuccess) {  // the tables above go out of scope
+            c->err = "upload of the sweep tables failed";
+            return bail(VEGAS_ECUDA);
         }
     }
     // ---- cooperative sweep: one sample, every block on every class

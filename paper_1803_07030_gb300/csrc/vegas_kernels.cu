@@ -1775,12 +1775,27 @@ int launch_cluster(const ResidentArgs &a, int n_clusters, int cs, int threads, v
     return (int)cudaLaunchKernelEx(&cfg, select_cluster(threads, a.pol != nullptr, a.smem_sites > 0), a);
 }
 
+namespace {
+
+// Raises a kernel's dynamic shared-memory limit to the device's: the limit belongs to the kernel,
+// which contexts of other sizes launch too, so it is not set to one context's size. False when
+// `bytes` do not fit.
+template <typename F>
+bool raise_smem_limit(F k, size_t bytes) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+           cudaFuncGetAttributes(&fa, k) == cudaSuccess && bytes + fa.sharedSizeBytes <= (size_t)most &&
+           cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes) == cudaSuccess;
+}
+
+}  // namespace
+
 int cluster_capacity(int cs, int threads, bool pol, size_t smem_bytes) {
     ClusterFn k = select_cluster(threads, pol, smem_bytes > 0);
     if (cs > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
-    if (smem_bytes > 0 &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
-        return 0;
+    if (smem_bytes > 0 && !raise_smem_limit(k, smem_bytes)) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs);
     cfg.blockDim = dim3(threads >= 512 ? 512 : 256);
@@ -1802,11 +1817,8 @@ int resident_blocks_per_sm(int threads, bool pol, size_t smem_bytes) {
     const bool smem = smem_bytes > 0;
     const int nt = resident_threads(threads, smem);
     const ResFn k = select_resident(nt, pol, smem);
-    if (smem && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
-        return 0;
     // the form without anisotropy terms takes the same shared memory
-    if (smem && cudaFuncSetAttribute(select_resident(nt, pol, smem, false), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem_bytes) != cudaSuccess)
+    if (smem && (!raise_smem_limit(k, smem_bytes) || !raise_smem_limit(select_resident(nt, pol, smem, false), smem_bytes)))
         return 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, nt, smem_bytes);
     return nb > 0 ? nb : (smem ? 0 : 1);

@@ -1,4 +1,5 @@
-// Device pieces of the tiled sweeps: named barriers, mailbox words, the wait for them.
+// Device pieces of the sweeps with spins in shared memory: named barriers, mailbox words, spins and
+// rows of links.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -48,6 +49,33 @@ __device__ __forceinline__ uint64_t tile_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+
+// The spin of local site i: x and y as one 8-byte pair, z in an array of its own (two loads).
+__device__ __forceinline__ float4 loc_spin(const float *sp, int cap, int i) {
+    const float2 xy = ((const float2 *)sp)[i];
+    return make_float4(xy.x, xy.y, sp[2 * cap + i], 0.f);
+}
+__device__ __forceinline__ void loc_set(float *sp, int cap, int i, float x, float y, float z) {
+    ((float2 *)sp)[i] = make_float2(x, y);
+    sp[2 * cap + i] = z;
+}
+
+// A fixed row of W links: (local site | lower flag << 16, J) pairs, or with FMT 1 one word per link,
+// the pair's first word with J's index in the sample's table of exchange values from bit 17 on.
+template <int W, int FMT>
+struct TileRow {
+    int4 q[W / 2];
+    __device__ __forceinline__ int site(int j) const { return (j & 1 ? q[j / 2].z : q[j / 2].x) & 0xFFFF; }
+    __device__ __forceinline__ bool lower(int j) const { return ((j & 1 ? q[j / 2].z : q[j / 2].x) >> 16) != 0; }
+    __device__ __forceinline__ float J(int j, const float *) const { return __int_as_float(j & 1 ? q[j / 2].w : q[j / 2].y); }
+};
+template <int W>
+struct TileRow<W, 1> {
+    int2 q[W / 2];
+    __device__ __forceinline__ int site(int j) const { return (j & 1 ? q[j / 2].y : q[j / 2].x) & 0xFFFF; }
+    __device__ __forceinline__ bool lower(int j) const { return ((j & 1 ? q[j / 2].y : q[j / 2].x) & 0x10000) != 0; }
+    __device__ __forceinline__ float J(int j, const float *t) const { return t[(j & 1 ? q[j / 2].y : q[j / 2].x) >> 17]; }
+};
 
 }  // namespace
 }  // namespace vegas

@@ -105,6 +105,22 @@ struct Tile64Args {
 int tile64_shape(Tile64Args &a, const TileShape &s, TilePlan &p, std::vector<double> &J, size_t *smem);
 int launch_tile64(const Tile64Args &a, int threads, size_t smem, void *stream);
 
+// ---- batches with spins in shared memory (vegas_batch.cu)
+constexpr int kBatchThreads = 512;    // sweeping threads per block
+
+struct BatchArgs {
+    ResidentArgs r;
+    const void *rows;            // [global site][kEllRow]: (site of the sample | lower flag << 16, J)
+                                 // pairs, or words with J's index in codes from bit 17 on
+    const float *codes;          // [n_codes]
+    const int32_t *modes;        // [segment] 0: no link to a lower colour, 1: every link, 2: flagged
+    uint32_t rk0[10], rk1[10];   // Philox round keys
+    int32_t n_codes, cubic, clusters, part_off;
+};
+
+int batch_capacity(BatchArgs a, int cs, int sm_count);
+int launch_batch(BatchArgs a, int n, int cs, void *stream);  // n clusters of cs blocks; the CUDA error
+
 // Sweep of a.mcs MCS and their records; returns the CUDA error.
 int launch_tile(const TileArgs &a, int threads, size_t smem, void *stream);
 
