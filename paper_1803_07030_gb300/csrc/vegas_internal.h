@@ -388,6 +388,10 @@ void launch_run_ctrl(const RunState *run, unsigned long long loop_handle, void *
 // Copies the spins into the snapshot slot of the step that just ended (read from the run state).
 void launch_snapshot(const void *spins, void *snap, int64_t n16, const RunState *run, int grid, void *stream);
 
+// A run's records from [record][instance] to [instance][record]: (E, Mx, My, Mz) and counts.
+void launch_by_instance(const double *hist, const uint32_t *acc, double *hist_t, uint32_t *acc_t, int64_t n_inst,
+                        int64_t n_rec, void *stream);
+
 // Cooperative launch (all blocks co-resident); returns the CUDA error of the launch.
 int launch_coop(const CoopArgs &a, int grid, void *stream);
 int coop_blocks_per_sm(bool pol, int form, bool fp64);  // form: 6 (rows of six links), kEllRow (padded rows) or 0

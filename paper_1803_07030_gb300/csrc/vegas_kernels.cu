@@ -1660,6 +1660,22 @@ __global__ void snapshot_kernel(const uint4 *spins, uint4 *snap, int64_t n16, co
         dst[w] = spins[w];
 }
 
+__global__ void by_instance_kernel(const double4_32a *hist, const uint32_t *acc, double4_32a *hist_t, uint32_t *acc_t,
+                                   int64_t n_inst, int64_t n_rec) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_inst * n_rec; k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = k / n_inst, i = k - r * n_inst;
+        hist_t[i * n_rec + r] = hist[k];
+        acc_t[i * n_rec + r] = acc[k];
+    }
+}
+
+void launch_by_instance(const double *hist, const uint32_t *acc, double *hist_t, uint32_t *acc_t, int64_t n_inst,
+                        int64_t n_rec, void *stream) {
+    const int grid = (int)std::min<int64_t>((n_inst * n_rec + 255) / 256, 2048);
+    by_instance_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>((const double4_32a *)hist, acc, (double4_32a *)hist_t, acc_t,
+                                                               n_inst, n_rec);
+}
+
 void launch_snapshot(const void *spins, void *snap, int64_t n16, const RunState *run, int grid, void *stream) {
     snapshot_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>((const uint4 *)spins, (uint4 *)snap, n16, run);
 }
