@@ -1295,45 +1295,43 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         std::vector<int32_t> h_modes;
         if (c->batch_ok) {
             // the samples' exchange values, when they are few: rows are then words
-            auto code_of = [&](float v) {
-                size_t k = 0;
-                while (k < h_codes.size() && h_codes[k] != v) ++k;
-                if (k == h_codes.size()) h_codes.push_back(v);
-                return (uint32_t)k;
-            };
-            code_of(0.0f);  // padding
             for (int32_t s = 0; s < n_samples && h_codes.size() <= (size_t)kTileCodes; ++s)
-                for (const double v : L[(size_t)s].J) {
-                    code_of((float)v);
-                    if (h_codes.size() > (size_t)kTileCodes) break;
-                }
+                exchange_values(L[(size_t)s].J.data(), (int64_t)L[(size_t)s].J.size(), h_codes);
             const bool words = h_codes.size() <= (size_t)kTileCodes;
             const int per = words ? 1 : 2;
             h_rows.resize((size_t)n_sites * kEllRow * per);
             BatchArgs &ba = c->batch;
             ba = BatchArgs{};
-            for (int32_t s = 0; s < n_samples; ++s) {
-                const LoadedSample &l = L[(size_t)s];
-                const SampleInfo &si = c->samples[(size_t)s];
+            for (const LoadedSample &l : L)
                 for (double x : l.k_cub) ba.cubic |= x != 0.0 ? 1 : 0;
-                for (int32_t q = 0; q < l.n_colours; ++q)
-                    for (int32_t g = l.cstart[(size_t)q]; g < l.cstart[(size_t)q + 1]; ++g) {
-                        uint32_t *row = &h_rows[(size_t)(si.site_off + g) * kEllRow * per];
-                        const int64_t e0 = l.row_ptr[(size_t)g], deg = l.row_ptr[(size_t)g + 1] - e0;
-                        for (int w = 0; w < kEllRow; ++w) {
-                            const bool in = w < deg;
-                            const int32_t j = in ? l.col[(size_t)(e0 + w)] : g;
-                            const float J = in ? (float)l.J[(size_t)(e0 + w)] : 0.0f;
-                            const uint32_t link = (uint32_t)j | (in && j < l.cstart[(size_t)q] ? 0x10000u : 0u);
-                            if (words) {
-                                row[w] = link | code_of(J) << 17;
-                            } else {
-                                row[2 * w] = link;
-                                row[2 * w + 1] = (uint32_t)float_bits(J);
-                            }
+            auto write_rows = [&](int64_t s) {
+                const LoadedSample &l = L[(size_t)s];
+                int32_t q = 0;
+                uint32_t code = 0;
+                for (int32_t g = 0; g < l.n; ++g) {
+                    while (g >= l.cstart[(size_t)q + 1]) ++q;
+                    uint32_t *row = &h_rows[(size_t)(c->samples[(size_t)s].site_off + g) * kEllRow * per];
+                    const int64_t e0 = l.row_ptr[(size_t)g], deg = l.row_ptr[(size_t)g + 1] - e0;
+                    for (int w = 0; w < kEllRow; ++w) {
+                        const bool in = w < deg;
+                        const int32_t j = in ? l.col[(size_t)(e0 + w)] : g;
+                        const float J = in ? (float)l.J[(size_t)(e0 + w)] : 0.0f;
+                        const uint32_t link = (uint32_t)j | (in && j < l.cstart[(size_t)q] ? 0x10000u : 0u);
+                        if (words) {
+                            if (h_codes[code] != J)
+                                for (code = 0; h_codes[code] != J; ++code) {}
+                            row[w] = link | code << 17;
+                        } else {
+                            row[2 * w] = link;
+                            row[2 * w + 1] = (uint32_t)float_bits(J);
                         }
                     }
-            }
+                }
+            };
+            host_ranges(n_samples, (int32_t)std::min<int64_t>({16, n_samples, n_sites / 32768 + 1}),
+                        [&](int64_t s0, int64_t s1) {
+                            for (int64_t s = s0; s < s1; ++s) write_rows(s);
+                        });
             for (const PassLaunch &pl : c->passes) h_modes.push_back(pl.args.lower_mode);  // segments are the passes in order
             ba.cubic = ba.cubic ? 1 : 0;
             ba.n_codes = words ? (int32_t)h_codes.size() : 0;
@@ -2005,14 +2003,18 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                     // The tiled form runs several times faster than any sweep timed above wherever it
                     // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 29, 55; 32^3 x
                     // 32 replicas 12, 38; the 29k-site core/shell particle 4.9, 23; a 13k-site fcc sphere
-                    // x 8 5.4, 24; 512 sites 2.1, 9), so it is not timed. It takes over where it adds the
+                    // x 8 5.4, 24; 512 sites 2.1, 9), so it is not timed: the cooperative form's time stands
+                    // for it, at 4/7 (the least gain measured, 29 to 55, with the probes' noise; the fcc
+                    // spheres: 15.6 us in clusters beside 24 and 5.4). It takes over where it adds the
                     // attempts' FP32 shares in the order of the sweep that would run (one thread per
                     // site of a class: the cooperative form, and every sweep of classes of at most 512
                     // sites) or where that order is not fixed anyway (the kernel of 32 replicas draws its
                     // blocks from a counter); elsewhere records would differ by the FP32 sums' rounding,
                     // 1e-9 of their norm.
                     if (c->tile_ok && !c->opt.resident_smem &&
-                        (best_v == 2 || c->max_class_sites <= kTileThreads ||
+                        (best_v == 2 ||
+                         (c->tune_ms[2] > 0.0 && c->tune_ms[2] * probe <= 1.75 * best) ||
+                         c->max_class_sites <= kTileThreads ||
                          (best_v == 0 && pass32_kind(c->passes[0].args) == VEGAS_KERNEL_PASS32_R32))) {
                         c->variant = best_v = 2;
                         best_c = Cand{2, 2, 0, 0, 0};

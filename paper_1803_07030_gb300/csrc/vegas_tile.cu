@@ -486,23 +486,29 @@ bool tile_plan(const TileShape &s, TilePlan &out) {
     return out.max_loc <= 65535;
 }
 
-namespace {
+void host_ranges(int64_t n, int32_t chunks, const std::function<void(int64_t, int64_t)> &f) {
+    if (n < 1) return;
+    if (chunks <= 1) return f(0, n);
+    for_parts(chunks, chunks * 4096, [&](int32_t q, uint32_t *) { f(n * q / chunks, n * (q + 1) / chunks); });
+}
 
-// The exchange values of the sample, as far as kTileCodes goes; padding adds 0.
-void exchange_values(const TileShape &s, std::vector<float> &values) {
-    const int64_t n_links = s.row_ptr[s.n];
-    const int32_t chunks = (int32_t)std::min<int64_t>(64, n_links / 4096 + 1);
-    std::vector<std::vector<float>> got((size_t)chunks);
+void exchange_values(const double *J, int64_t n_links, std::vector<float> &values) {
     auto add = [](std::vector<float> &to, float v) {
         if (to.size() <= (size_t)kTileCodes && std::find(to.begin(), to.end(), v) == to.end()) to.push_back(v);
     };
-    for_parts(chunks, chunks * 4096, [&](int32_t q, uint32_t *) {
-        for (int64_t e = n_links * q / chunks; e < n_links * (q + 1) / chunks; ++e) add(got[(size_t)q], (float)s.J[e]);
-    });
+    auto scan = [&](std::vector<float> &to, int64_t e0, int64_t e1) {
+        for (int64_t e = e0; e < e1; ++e)
+            if (e == e0 || J[e] != J[e - 1]) add(to, (float)J[e]);
+    };
+    const int32_t chunks = (int32_t)std::min<int64_t>(16, n_links / (1 << 19) + 1);  // a thread costs 0.05 ms
+    std::vector<std::vector<float>> got((size_t)chunks);
+    host_ranges(chunks, chunks, [&](int64_t q, int64_t) { scan(got[(size_t)q], n_links * q / chunks, n_links * (q + 1) / chunks); });
     for (const auto &x : got)
         for (float v : x) add(values, v);
     add(values, 0.0f);
 }
+
+namespace {
 
 // The block's tables: sites, ids, words, and the rows in local site numbers, as pairs or
 // (a.n_codes) words.
@@ -525,6 +531,7 @@ void write_tables(const TileArgs &a, const TileShape &s, TilePlan &p) {
             p.halo_slot[(size_t)(pt.halo_begin + h)] = p.parts[(size_t)p.part[(size_t)g]].word_begin + p.word[(size_t)g];
         }
         int c = 0;
+        uint32_t code = 0;
         for (int32_t k = 0; k < pt.n_own; ++k) {
             while (k >= p.classes[(size_t)q * a.n_colours + c].end) ++c;
             const int32_t g = own[(size_t)k], w0 = p.word[(size_t)g];
@@ -542,8 +549,8 @@ void write_tables(const TileArgs &a, const TileShape &s, TilePlan &p) {
                     J = (float)s.J[e0 + w];
                 }
                 if (a.n_codes) {
-                    uint32_t code = 0;
-                    while (p.codes[code] != J) ++code;
+                    if (p.codes[code] != J)
+                        for (code = 0; p.codes[code] != J; ++code) {}
                     ((uint32_t *)p.rows.get())[at + w] = link | code << 17;
                 } else {
                     int2 x = make_int2((int)link, 0);
@@ -598,7 +605,7 @@ int tile_shape(TileArgs &a, const TileShape &s, TilePlan &p, size_t *smem) {
     const int best = std::min(kTileThreads, std::max({64, ((own + rounds - 1) / rounds + 31) / 32 * 32, (halo / 2 + 31) / 32 * 32}));
     cudaFuncAttributes rec;  // loads the record kernel now, not in the first (timed) launch
     if (cudaFuncGetAttributes(&rec, tile_record_kernel) != cudaSuccess) return 0;
-    exchange_values(s, p.codes);
+    exchange_values(s.J, s.row_ptr[s.n], p.codes);
     const bool words = p.codes.size() <= (size_t)kTileCodes && !a.pass.pol32 && !a.cubic;
     // pairs in shared memory, then words there, then words (or pairs) through L1
     int found = 0;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <functional>
 #include <memory>
 #include <vector>
 
@@ -75,6 +76,10 @@ struct TilePlan {
     bool columns = false;
 };
 
+// Adds the exchange values J[0..n), as far as kTileCodes goes, and padding's 0.
+void exchange_values(const double *J, int64_t n, std::vector<float> &values);
+// f(begin, end) for the chunks of [0, n), on several host threads.
+void host_ranges(int64_t n, int32_t chunks, const std::function<void(int64_t, int64_t)> &f);
 // False when the sample cannot be cut so.
 bool tile_plan(const TileShape &s, TilePlan &out);
 // Chooses the threads per block and what it keeps in shared memory, and writes the rows; 0 when
