@@ -510,9 +510,10 @@ int32_t vegas_greedy_colour(int32_t n_sites, const int64_t *row_ptr, const int32
  * replaced, e.g. by cudaDeviceReset) looks up the device address of the static scratch
  * (cudaGetSymbolAddress) with that device current; make that first call before any stream
  * capture begins. Blocking: every call waits for the sweep to finish on `stream` and reads
- * the error word back with a blocking copy before it returns. Every call uses the same
- * scratch and rewrites it; calls whose GPU work overlaps (other threads, other streams)
- * race on it. Errors: VEGAS_EINVAL for bad sizes, NULL or misaligned pointers (message from
+ * the error word before it returns. Calls with classes of at most 8192 attempts (sites x
+ * replicas) are one launch that needs no scratch, on GPUs that read ordinary host memory;
+ * the others use the same scratch and rewrite it, and such calls whose GPU work overlaps
+ * (other threads, other streams) race on it. Errors: VEGAS_EINVAL for bad sizes, NULL or misaligned pointers (message from
  * vegas_noalloc_last_error), VEGAS_ECUDA, VEGAS_EDEVICE (1: NaN energy change; 4: a bad
  * index seen by a debug build).
  */

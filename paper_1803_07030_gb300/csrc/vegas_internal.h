@@ -388,6 +388,29 @@ void launch_run_ctrl(const RunState *run, unsigned long long loop_handle, void *
 // Copies the spins into the snapshot slot of the step that just ended (read from the run state).
 void launch_snapshot(const void *spins, void *snap, int64_t n16, const RunState *run, int grid, void *stream);
 
+// One whole MCS on the caller's memory in one launch (vegas_sweep_noalloc): one thread-block
+// cluster takes the colour classes in turn.
+constexpr int kOnceThreads = 256;  // most threads per block
+constexpr int kOnceBlocks = 8;     // most blocks (the portable cluster size)
+// Most attempts of a class, four rounds of the cluster: a round of the two classes of a simple
+// cubic sample takes 3 us, one launch per class 26 us more than the one launch. Calls from
+// Python, one launch and one per class: 27 and 54 us up to 1000 sites, 39 and 56 at 8192
+// attempts per class, 52 and 56 at 16384, 108 and 62 at 55296.
+constexpr int64_t kOnceWork = 4 * kOnceThreads * kOnceBlocks;
+
+struct OnceArgs {
+    PassArgs pass;  // pointers, seed, ids, uniform parameters; no run state
+    uint32_t t;
+    int32_t n_colours;
+    int32_t cstart[kMaxColours + 1];
+    float beta[32], B[32];
+    double *out;    // [R][4]
+    uint32_t *err;  // written when an energy change is NaN; may be host memory
+};
+
+// For classes of at most `widest` attempts (site x replica). 0, or the launch's error.
+int launch_sweep_once(const OnceArgs &a, int64_t widest, void *stream);
+
 // A run's records from [record][instance] to [instance][record]: (E, Mx, My, Mz) and counts.
 void launch_by_instance(const double *hist, const uint32_t *acc, double *hist_t, uint32_t *acc_t, int64_t n_inst,
                         int64_t n_rec, void *stream);

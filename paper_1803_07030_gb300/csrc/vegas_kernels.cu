@@ -788,6 +788,59 @@ __global__ void __launch_bounds__(NT) resident32_kernel(const ResidentArgs a) {
     if (nan_seen) atomicOr(a.err, kErrNaN);
 }
 
+// ------------------------------------------------------------------ one MCS in one launch
+// One cluster sweeps the classes in turn, a cluster barrier after each, and adds the blocks' sums
+// in block 0's shared memory. Everything a call sets comes in the kernel's arguments, so no
+// launch has to write or clear a run state first. Neighbours are read through L2: other blocks
+// write them. A call is bound by latencies: the launch and the wait for it (about 10 us), then
+// per class row offsets, links and neighbours one after the other (the first row of the next
+// class is on its way to L1 before the barrier), 1.5 us. On 13 x 11 x 9 sites a call took 75 us
+// with a set-up launch, one per class, the reduction and a copy of the error word; 33 us now.
+template <int PM>
+__global__ void __launch_bounds__(kOnceThreads, 2) sweep_once_kernel(const __grid_constant__ OnceArgs o) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double s_sum[kOnceBlocks][32][4];  // block 0's: the blocks' sums
+    const PassArgs &a = o.pass;
+    const int rank = (int)cl.block_rank(), blocks = (int)cl.num_blocks();
+    const int R = 1 << a.log2R, n = blocks * blockDim.x, tid = rank * blockDim.x + threadIdx.x;
+    const int r = tid & (R - 1);  // n is a multiple of 32 >= R
+    const float beta = o.beta[r], B = o.B[r];
+    const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
+    const int2 *E = (const int2 *)a.edges;
+    const Site32 p = site_params32(a, PM, 0);
+    Acc32 acc;
+    bool nan_seen = false;
+    for (int c = 0; c < o.n_colours; ++c) {
+        const int g1 = o.cstart[c + 1];
+        for (int g = o.cstart[c] + (tid >> a.log2R); g < g1; g += n >> a.log2R) {
+            float4 Sq;
+            direct_attempt<PM, 2, 0, 1>((float4 *)a.spins, E, a.row_ptr, g, r, R, o.cstart[c], (uint32_t)__ldg(a.orig + g), p,
+                                        beta, B, o.t, (uint32_t)(a.inst0 + r), k0, k1, acc, nan_seen, nullptr, 0.f, Sq);
+            acc.flush();  // sums in FP64, whatever the number of attempts per thread
+        }
+        const int next = g1 + (tid >> a.log2R);
+        if (c + 1 < o.n_colours && next < o.cstart[c + 2]) {  // the next row, while the others finish
+            const int64_t e0 = __ldg(a.row_ptr + next), e1 = __ldg(a.row_ptr + next + 1);
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(a.orig + next));
+            if (e1 > e0) {
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(E + e0));
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(E + e1 - 1));
+            }
+        }
+        cl.sync();  // the class's spins are final, for the cluster
+    }
+    if (nan_seen) *(volatile uint32_t *)o.err = kErrNaN;
+    block_partials(acc.d, 0, R, cl.map_shared_rank(&s_sum[0][0][0], 0) + rank * 32 * 4, nullptr);
+    cl.sync();
+    if (rank == 0)
+        for (int k = threadIdx.x; k < R * 4; k += blockDim.x) {
+            double v = 0.0;
+            for (int b = 0; b < blocks; ++b) v += s_sum[b][k >> 2][k & 3];
+            o.out[k] = v;
+        }
+}
+
 // ------------------------------------------------------------------ cluster sweep
 // As the resident sweep, but a thread-block cluster of CS blocks (on CS SMs) takes each
 // instance: the blocks split every colour segment, meet at the hardware cluster barrier
@@ -1773,6 +1826,25 @@ size_t cluster_smem_bytes(const ResidentArgs &a, int threads) {
     // groups' regions start at even site counts (sm_spin's pairs stay 8-byte aligned)
     const int64_t sites = std::max<int64_t>(a.smem_sites, ng > 1 ? (int64_t)ng * ((a.group_sites + 1) & ~1) : 0);
     return (size_t)sites * 3 * sizeof(float);
+}
+
+int launch_sweep_once(const OnceArgs &a, int64_t widest, void *stream) {
+    // more blocks first, then longer ones: the SMs' latencies overlap (64 to 256 threads at first: the same)
+    int nt = 64, nb = 1;
+    while (nb < kOnceBlocks && (int64_t)nb * nt < widest) nb *= 2;
+    while (nt < kOnceThreads && (int64_t)nb * nt < widest) nt *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nb);
+    cfg.blockDim = dim3((unsigned)nt);
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)nb;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return (int)cudaLaunchKernelEx(&cfg, a.pass.params_mode ? sweep_once_kernel<1> : sweep_once_kernel<0>, a);
 }
 
 int launch_cluster(const ResidentArgs &a, int n_clusters, int cs, int threads, void *stream) {

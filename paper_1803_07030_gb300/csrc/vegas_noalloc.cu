@@ -86,6 +86,7 @@ __global__ void noalloc_setup(const SetupArgs s) {
 struct ScratchSlot {
     unsigned long long ctx_id;  // 0: not looked up yet
     void *addr;
+    int host_access;  // the GPU reads and writes ordinary host memory
 };
 std::mutex g_mu;
 ScratchSlot g_slot[kNoAllocMaxDevices] = {};
@@ -123,6 +124,13 @@ unsigned long long current_context_id() {
 vegas_status fail(vegas_status st, const std::string &m) {
     g_err = m;
     return st;
+}
+
+vegas_status sweep_status(uint32_t err) {
+    if (err)
+        return fail(VEGAS_EDEVICE, "device error flags " + std::to_string(err) +
+                                       " (1: NaN energy change, 4: bad row or neighbour index seen by a debug build)");
+    return VEGAS_OK;
 }
 
 // A host exception caught at the entry point, as a status (called inside a catch block).
@@ -168,6 +176,7 @@ extern "C" vegas_status vegas_sweep_noalloc(void *spins, const void *links, cons
         if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
         if (dev < 0 || dev >= kNoAllocMaxDevices) return fail(VEGAS_EINVAL, "device ordinal too large");
         void *base = nullptr;
+        bool host_access = false;
         {
             // set-up, once per device and CUDA context, with the device current: the device
             // address of the static scratch (in host code its name is only a host-side handle)
@@ -178,20 +187,20 @@ extern "C" vegas_status vegas_sweep_noalloc(void *spins, const void *links, cons
                 void *addr = nullptr;
                 e = cudaGetSymbolAddress(&addr, g_noalloc_scratch);
                 if (e != cudaSuccess) {
-                    sl = ScratchSlot{0, nullptr};
+                    sl = ScratchSlot{0, nullptr, 0};
                     return fail(VEGAS_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
                 }
                 if (id == 0) id = current_context_id();  // the lookup made the primary context current
-                sl = ScratchSlot{id, addr};
+                int pageable = 0;
+                if (cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess) pageable = 0;
+                sl = ScratchSlot{id, addr, pageable};
             }
             base = sl.addr;
+            host_access = sl.host_access != 0;
         }
         NoAllocHeader *hdr = (NoAllocHeader *)base;
         double *partial = (double *)((unsigned char *)base + kHeaderBytes);
 
-        int sm = 0;
-        e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
         int log2R = 0;
         while ((1 << log2R) < replicas) ++log2R;
 
@@ -227,7 +236,38 @@ extern "C" vegas_status vegas_sweep_noalloc(void *spins, const void *links, cons
         a.u32 = SiteParams32{(float)p[0], (float)p[1], (float)p[2], (float)p[3], (float)p[4],
                              (float)p[5], (float)p[6], (float)p[7], (float)p[8]};
         a.u64 = SiteParams64{p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]};
+        cudaStream_t st = (cudaStream_t)stream;
         const int per_class = std::max(1, kNoAllocMaxBlocks / n_colours);
+#ifndef VEGAS_DEBUG_CHECKS
+        int64_t widest = 1;
+        for (int c = 0; c < n_colours; ++c)
+            widest = std::max(widest, (int64_t)(colour_start[c + 1] - colour_start[c]) << log2R);
+        if (widest <= kOnceWork && host_access) {
+            thread_local uint32_t err_word;  // the kernel writes it only to report an error
+            err_word = 0;
+            OnceArgs oa;
+            std::memset(&oa, 0, sizeof oa);
+            oa.pass = a;
+            oa.t = t;
+            oa.n_colours = n_colours;
+            std::memcpy(oa.cstart, colour_start, sizeof(int32_t) * (n_colours + 1));
+            for (int r = 0; r < replicas; ++r) {
+                oa.beta[r] = (float)beta[r];
+                oa.B[r] = (float)field[r];
+            }
+            oa.out = out;
+            oa.err = &err_word;
+            if (launch_sweep_once(oa, widest, st) == cudaSuccess) {
+                e = cudaStreamSynchronize(st);
+                if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("sweep: ") + cudaGetErrorString(e));
+                return sweep_status(*(volatile uint32_t *)&err_word);
+            }
+            cudaGetLastError();  // no such cluster: class by class
+        }
+#endif
+        int sm = 0;
+        e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
         const int occ = sm * pass_blocks_per_sm(32, a);
         int grids[kMaxColours];
         int total = 0;
@@ -250,7 +290,6 @@ extern "C" vegas_status vegas_sweep_noalloc(void *spins, const void *links, cons
             sa.beta[r] = beta[r];
             sa.B[r] = field[r];
         }
-        cudaStream_t st = (cudaStream_t)stream;
         noalloc_setup<<<1, 32, 0, st>>>(sa);
         int slot = 0;
         for (int c = 0; c < n_colours; ++c) {  // an empty class runs one block that writes zeros
@@ -270,10 +309,7 @@ extern "C" vegas_status vegas_sweep_noalloc(void *spins, const void *links, cons
         uint32_t err = 0;
         e = cudaMemcpy(&err, hdr->err, sizeof err, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("error word: ") + cudaGetErrorString(e));
-        if (err)
-            return fail(VEGAS_EDEVICE, "device error flags " + std::to_string(err) +
-                                           " (1: NaN energy change, 4: bad row or neighbour index seen by a debug build)");
-        return VEGAS_OK;
+        return sweep_status(err);
     } catch (...) {
         return noalloc_host_exception();
     }
