@@ -160,6 +160,11 @@ struct vegas_ctx {
     int32_t *d_tasks = nullptr;
     int32_t *d_deps = nullptr;  // wavefront sweep: distinct class-0 blocks of each class-1 block
     std::vector<LaunchGroup> launches;  // the per-class sweep's launches of one MCS, in class order
+    // samples whose passes all run as the R = 32 kernel, which keeps each site's 32 spins in planes
+    std::vector<char> planar_ok;  // per sample
+    int n_planar = 0;
+    bool planar = false;          // those samples' rows are in planes now
+    uint8_t *d_planar_site = nullptr;  // [global site] when some samples are and some are not
     // renormalisation folded into the step's last class-1 pass (per-class sweep, R = 32)
     bool fold_ok = false;
     PassArgs fold_args{};       // the class-1 pass's arguments with the fold's fields
@@ -241,7 +246,7 @@ void free_all(vegas_ctx *c) {
                     c->d_insts, c->d_cstart, c->d_queue, c->d_bar, c->d_coop_partial, c->d_acc, c->d_acc_hist,
                     c->d_pol, c->d_pol32, c->d_qis, c->d_sigma, c->d_adapt_n, c->d_type_hist, c->d_snap, c->d_segs,
                     c->d_tasks, c->d_deps, c->d_done, c->d_ticket, c->d_pass_tickets, c->d_wave_partial, c->d_wave_slot_base, c->d_wave_slot_count,
-                    c->d_fold_deps, c->d_fold_deg, c->d_fold_cnt};
+                    c->d_fold_deps, c->d_fold_deg, c->d_fold_cnt, c->d_planar_site};
     for (void *b : bufs)
         if (b) cudaFree(b);
     for (void *b : c->tile_bufs) cudaFree(b);
@@ -454,10 +459,31 @@ int enqueue_wave(vegas_ctx *c, cudaStream_t st) {
     return e;
 }
 
+// Whether the sweep of variant v keeps rows in planes, and the rows of those samples so (or not).
+bool planar_for(const vegas_ctx *c, int v) { return v == 0 && c->n_planar > 0; }
+void set_planar(vegas_ctx *c, bool want) {
+    if (c->planar == want) return;
+    for (int32_t s = 0; s < c->n_samples; ++s) {
+        if (!c->planar_ok[(size_t)s]) continue;
+        const SampleInfo &si = c->samples[(size_t)s];
+        const int grid = (int)std::min<int64_t>((si.n + 7) / 8, (int64_t)c->sm_count * 8);
+        launch_planar(c->d_spins, si.site_off, (int64_t)si.site_off + si.n, want, grid, c->stream);
+        c->kernel_launches++;
+    }
+    c->planar = want;
+}
+
 // Renormalisation at the end of a step (unless the step's last pass did it: folded), then
 // (option snapshots) the copy of the final state.
 void enqueue_renorm(vegas_ctx *c, cudaStream_t st, bool folded = false) {
-    RenormArgs ra{c->d_spins, c->d_norm, c->n_sites * c->R, c->log2R, c->d_qis};
+    RenormArgs ra{};
+    ra.spins = c->d_spins;
+    ra.norm = c->d_norm;
+    ra.n_work = c->n_sites * c->R;
+    ra.log2R = c->log2R;
+    ra.qis = c->d_qis;
+    if (planar_for(c, c->variant)) ra.planar = c->n_planar == c->n_samples ? 1 : 2;
+    ra.planar_site = c->d_planar_site;
     const int grid = (int)std::min<int64_t>((ra.n_work + 255) / 256, (int64_t)c->sm_count * 8);
     if (c->precision == 64)
         launch_renorm64(ra, grid, st);
@@ -1486,6 +1512,26 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         ca.ell = use_ell ? c->d_ell : nullptr;
         c->coop_eligible = true;
     }
+    // ---- rows in planes: the samples whose every pass runs as the R = 32 kernel (use of it is
+    // decided by the rows and the options, so all passes of a sample agree)
+    c->planar_ok.assign((size_t)n_samples, 0);
+    if (c->precision == 32 && c->R == 32) {
+        for (auto &x : c->planar_ok) x = 1;
+        for (const PassLaunch &pl : c->passes)
+            if (!pass32_r32_rows(pl.args)) c->planar_ok[(size_t)pl.sample] = 0;
+        for (char x : c->planar_ok) c->n_planar += x;
+        if (c->n_planar > 0 && c->n_planar < n_samples) {
+            std::vector<uint8_t> site((size_t)n_sites, 0);
+            for (int32_t s = 0; s < n_samples; ++s)
+                if (c->planar_ok[(size_t)s])
+                    std::fill_n(site.begin() + c->samples[(size_t)s].site_off, c->samples[(size_t)s].n, (uint8_t)1);
+            DALLOC(c->d_planar_site, site.size());
+            if (cudaMemcpy(c->d_planar_site, site.data(), site.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+                c->err = "upload of the row forms failed";
+                return bail(VEGAS_ECUDA);
+            }
+        }
+    }
     // ---- renormalisation folded into the step's last class-1 pass: one sample of two colour
     // classes swept by the R = 32 kernel without a policy table (every class-1 link to class 0),
     // no discrete-valued sites, every class-0 block read by some class-1 block
@@ -1976,6 +2022,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                         if (v == 2) set_coop_shape(c, vc.a);
                         if (v == 3 && !set_cluster_shape(c, vc.a, vc.b, vc.split, vc.group, vc.group * 16, vc.sm != 0))
                             continue;
+                        set_planar(c, planar_for(c, v));
                         cudaEvent_t x0, x1;
                         CK(c, cudaEventCreate(&x0));
                         CK(c, cudaEventCreate(&x1));
@@ -2035,6 +2082,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                 c->tuned = true;
             }
 
+            set_planar(c, planar_for(c, c->variant));
             if (m0 == 0 && c->tuned && use_graph && c->opt.graphs == 1 && step_graph_nodes(c, mcs) > 0) {
                 // every remaining step in one launch of the run graph
                 cudaGraphExec_t ge;
@@ -2153,7 +2201,13 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                                 std::memcpy(o3, p, 3 * sizeof(double));
                             } else {
                                 float f[3];
-                                std::memcpy(f, p, sizeof f);
+                                if (c->planar && c->planar_ok[(size_t)sm]) {  // (x, y) pairs, then z
+                                    const unsigned char *row = p - (size_t)r * vbytes;
+                                    std::memcpy(f, row + (size_t)r * 8, 8);
+                                    std::memcpy(f + 2, row + 256 + (size_t)r * 4, 4);
+                                } else {
+                                    std::memcpy(f, p, sizeof f);
+                                }
                                 for (int q = 0; q < 3; ++q) o3[q] = f[q];
                             }
                         }
@@ -2346,13 +2400,14 @@ vegas_status spins_io(vegas_ctx *c, int32_t inst, double *out, const double *in)
     const SampleInfo &si = c->samples[(size_t)(inst / c->R)];
     const int32_t r = inst % c->R;
     const size_t n = (size_t)si.n;
+    const bool planar = c->planar && c->planar_ok[(size_t)(inst / c->R)];
     double *d = nullptr;
     CK(c, cudaMalloc(&d, sizeof(double) * 3 * n));
     std::vector<double> h(3 * n);
     const int grid = (int)std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)c->sm_count * 8);
     cudaError_t e = cudaSuccess;
     if (out) {
-        launch_gather(c->d_spins, c->precision, si.site_off, (int64_t)n, c->log2R, r, d, grid, c->stream);
+        launch_gather(c->d_spins, c->precision, si.site_off, (int64_t)n, c->log2R, r, planar, d, grid, c->stream);
         e = cudaMemcpyAsync(h.data(), d, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e == cudaSuccess)
@@ -2369,7 +2424,7 @@ vegas_status spins_io(vegas_ctx *c, int32_t inst, double *out, const double *in)
                 h[3 * g + q] = v;
             }
         e = cudaMemcpyAsync(d, h.data(), sizeof(double) * 3 * n, cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) launch_scatter(c->d_spins, c->precision, si.site_off, (int64_t)n, c->log2R, r, d, grid, c->stream);
+        if (e == cudaSuccess) launch_scatter(c->d_spins, c->precision, si.site_off, (int64_t)n, c->log2R, r, planar, d, grid, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     }
     c->kernel_launches++;

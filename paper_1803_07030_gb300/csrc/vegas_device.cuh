@@ -33,6 +33,19 @@ __device__ __forceinline__ float cub32(float x, float y, float z) {
     return fmaf(xx, yy, fmaf(yy, zz, xx * zz));
 }
 
+// ------------------------------------------------------------------ rows of 32 replicas
+// A site's 32 spins in planes: 32 (x, y) pairs, then 32 z (384 bytes; in memory each site keeps
+// the 512 bytes that 32 float4 take, so rows change their form in place).
+constexpr int kPlanarRow = 96;  // floats
+__device__ __forceinline__ float4 planar_spin(const float *row, int r) {
+    const float2 xy = ((const float2 *)row)[r];
+    return make_float4(xy.x, xy.y, row[64 + r], 0.f);
+}
+__device__ __forceinline__ void planar_set(float *row, int r, float4 v) {
+    ((float2 *)row)[r] = make_float2(v.x, v.y);
+    row[64 + r] = v.z;
+}
+
 // ------------------------------------------------------------------ block partials
 // Per-block sums of (E, Mx, My, Mz) for each replica. Lanes whose index agrees modulo R
 // hold the same replica; a fixed butterfly and a fixed warp order make the result

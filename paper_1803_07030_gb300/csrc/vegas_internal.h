@@ -190,6 +190,7 @@ struct PassArgs {
     int32_t depth;             // staged FP32 kernel: cp.async pipeline depth (2..4); 0 = direct kernel
     uint32_t *ticket;          // R = 32 staged kernel: next block of 8 sites of this pass (zeroed
                                // by the MCS's reduction); unused by the other kernels
+    uint32_t rk0[10], rk1[10]; // R = 32 staged kernel: Philox round keys (set at the launch)
     int32_t pol_fixed;         // FP32 with a policy table: the one policy of every site of the
                                // pass, or -1 (mixed, or no table)
     // The step's last class-1 pass of a two-class sample (R = 32 kernel) with the
@@ -225,6 +226,8 @@ struct RenormArgs {
     const double *norm;      // [global site] spin norm s_i
     int64_t n_work;          // global sites * R
     int32_t log2R;
+    int32_t planar;          // FP32 rows of 32 replicas: 0 float4, 1 planes, 2 by site
+    const uint8_t *planar_site;  // [global site], with 2
     const int32_t *qis;      // [global site] 1 for qIsing sites (left as they are), or NULL
 };
 
@@ -363,6 +366,7 @@ uint32_t pass32_kind(const PassArgs &a);
 PassFn select_direct(int pm, int lm, bool pol);
 
 // Sweep launch of one colour class; lower_mode, params_mode and deg pick the compiled variant.
+bool pass32_r32_rows(const PassArgs &a);  // the R = 32 kernel runs the pass: rows in planes
 void launch_pass32(const PassArgs &a, int grid, void *stream);
 void launch_pass64(const PassArgs &a, int grid, int threads, void *stream);  // threads: 32 .. kThreads
 void launch_reduce(const ReduceArgs &a, void *stream);
@@ -370,10 +374,12 @@ void launch_renorm32(const RenormArgs &a, int grid, void *stream);
 void launch_renorm64(const RenormArgs &a, int grid, void *stream);
 void launch_init32(const InitArgs &a, int grid, void *stream);
 void launch_init64(const InitArgs &a, int grid, void *stream);
-void launch_gather(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r, double *out3,
-                   int grid, void *stream);
+// The rows of sites [begin, end) (32 replicas, FP32) to planes or back.
+void launch_planar(void *spins, int64_t begin, int64_t end, bool to_planar, int grid, void *stream);
+void launch_gather(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r, bool planar,
+                   double *out3, int grid, void *stream);
 void launch_scatter(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r,
-                    const double *in3, int grid, void *stream);
+                    bool planar, const double *in3, int grid, void *stream);
 
 // Blocks per SM the pass kernels reach at kThreads threads (occupancy query).
 int pass_blocks_per_sm(int precision, const PassArgs &a);

@@ -1532,8 +1532,15 @@ __global__ void renorm64_kernel(const RenormArgs a) {
 __global__ void renorm32_kernel(const RenormArgs a) {
     float4 *S = (float4 *)a.spins;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < a.n_work; w += (int64_t)gridDim.x * blockDim.x) {
-        if (a.qis && a.qis[w >> a.log2R]) continue;  // discrete values keep their length
-        S[w] = renorm_spin32(S[w], a.norm[w >> a.log2R]);
+        const int64_t g = w >> a.log2R;
+        if (a.qis && a.qis[g]) continue;  // discrete values keep their length
+        if (a.planar == 1 || (a.planar == 2 && a.planar_site[g])) {
+            float *row = (float *)(S + g * 32);
+            const int r = (int)(w & 31);
+            planar_set(row, r, renorm_spin32(planar_spin(row, r), a.norm[g]));
+        } else {
+            S[w] = renorm_spin32(S[w], a.norm[g]);
+        }
     }
 }
 
@@ -1580,9 +1587,25 @@ __global__ void init_kernel(const InitArgs a) {
     }
 }
 
+// ------------------------------------------------------------------ rows of 32 replicas
+// Rows of sites [begin, end) from 32 float4 to planes or back, in place: one warp per row.
+__global__ void planar_kernel(float4 *S, int64_t begin, int64_t end, int to_planar) {
+    const int r = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t g = begin + (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < end; g += warps) {
+        float4 *row = S + g * 32;
+        const float4 v = to_planar ? row[r] : planar_spin((const float *)row, r);
+        __syncwarp();  // the whole row is read before any of it is written
+        if (to_planar)
+            planar_set((float *)row, r, v);
+        else
+            row[r] = v;
+    }
+}
+
 // ------------------------------------------------------------------ gather / scatter
 __global__ void gather_kernel(const void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r,
-                              double *out) {
+                              int planar, double *out) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t w = ((site_off + i) << log2R) + r;
         if (precision == 64) {
@@ -1591,7 +1614,8 @@ __global__ void gather_kernel(const void *spins, int precision, int64_t site_off
             out[3 * i + 1] = v.y;
             out[3 * i + 2] = v.z;
         } else {
-            const float4 v = ((const float4 *)spins)[w];
+            const float4 v = planar ? planar_spin((const float *)((const float4 *)spins + (site_off + i) * 32), r)
+                                    : ((const float4 *)spins)[w];
             out[3 * i] = v.x;
             out[3 * i + 1] = v.y;
             out[3 * i + 2] = v.z;
@@ -1600,13 +1624,18 @@ __global__ void gather_kernel(const void *spins, int precision, int64_t site_off
 }
 
 __global__ void scatter_kernel(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r,
-                               const double *in) {
+                               int planar, const double *in) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t w = ((site_off + i) << log2R) + r;
         if (precision == 64)
             ((double4_32a *)spins)[w] = make_double4_32a(in[3 * i], in[3 * i + 1], in[3 * i + 2], 0.0);
-        else
-            ((float4 *)spins)[w] = make_float4((float)in[3 * i], (float)in[3 * i + 1], (float)in[3 * i + 2], 0.f);
+        else {
+            const float4 v = make_float4((float)in[3 * i], (float)in[3 * i + 1], (float)in[3 * i + 2], 0.f);
+            if (planar)
+                planar_set((float *)((float4 *)spins + (site_off + i) * 32), r, v);
+            else
+                ((float4 *)spins)[w] = v;
+        }
     }
 }
 
@@ -1650,7 +1679,12 @@ void launch_pass32_multi(const PassArgs &key, const PassArgs *passes, const int3
 }
 
 void launch_pass32(const PassArgs &a, int grid, void *stream) {
-    select_pass32(a)<<<grid, pass32_threads(a), pass32_smem(a), (cudaStream_t)stream>>>(a);
+    PassArgs b = a;
+    for (uint32_t q = 0; q < 10; ++q) {
+        b.rk0[q] = (uint32_t)a.seed + q * 0x9E3779B9u;
+        b.rk1[q] = (uint32_t)(a.seed >> 32) + q * 0xBB67AE85u;
+    }
+    select_pass32(a)<<<grid, pass32_threads(a), pass32_smem(a), (cudaStream_t)stream>>>(b);
 }
 
 void launch_pass64(const PassArgs &a, int grid, int threads, void *stream) {
@@ -1677,14 +1711,18 @@ void launch_init64(const InitArgs &a, int grid, void *stream) {
     init_kernel<double4_32a><<<grid, 256, 0, (cudaStream_t)stream>>>(a);
 }
 
-void launch_gather(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r, double *out3,
-                   int grid, void *stream) {
-    gather_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(spins, precision, site_off, n, log2R, r, out3);
+void launch_planar(void *spins, int64_t begin, int64_t end, bool to_planar, int grid, void *stream) {
+    planar_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>((float4 *)spins, begin, end, to_planar ? 1 : 0);
+}
+
+void launch_gather(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r, bool planar,
+                   double *out3, int grid, void *stream) {
+    gather_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(spins, precision, site_off, n, log2R, r, planar, out3);
 }
 
 void launch_scatter(void *spins, int precision, int64_t site_off, int64_t n, int32_t log2R, int32_t r,
-                    const double *in3, int grid, void *stream) {
-    scatter_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(spins, precision, site_off, n, log2R, r, in3);
+                    bool planar, const double *in3, int grid, void *stream) {
+    scatter_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(spins, precision, site_off, n, log2R, r, planar, in3);
 }
 
 __global__ void advance_kernel(RunState *run, int32_t n) {

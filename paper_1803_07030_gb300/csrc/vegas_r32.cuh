@@ -25,15 +25,23 @@ namespace {
 // POL = 1 adds the sites' update policies (8 bytes each, staged with the caller ids); POL =
 // 2 + c does the same for a pass whose sites all have policy c, with the trial of that policy
 // alone compiled in (each site's parameter still comes from its entry).
-// Without a policy table the kernel runs in blocks of 7 warps, four blocks per SM (72
-// registers, 56 KB of shared memory each: 28 warps per SM); with one, in blocks of 8 warps,
-// three per SM. The block's partial sums are formed in each warp's own shared-memory area
-// once its sweep is done, so the block needs no other shared memory.
+// Rows are kept in planes (384 bytes of a site's 512): what the kernel moves most. A site's seven
+// rows come as 168 16-byte pieces, lane + 32 i the i-th of a lane. Per launch on 128^3 sites x 32,
+// against rows of 32 float4: 1.23 GB of DRAM traffic against 1.48, 217 M warp instructions
+// against 211, issue 70% against 61, 254 us against 274; on 256^3 1.95 ms against 2.04. It is now
+// bound by issue and the shared-memory pipe (61%) more than by DRAM (61%). The Philox round keys
+// are kernel arguments, which frees 20 registers; yet 24 warps per SM (8 x 3) stay the best:
+// 513 us per MCS on 128^3, 28 warps 522, 32 warps 544, 36 warps 567, 16 warps 567. Also tried:
+// alternate directions of the passes, so that one starts where the other ended in L2 (no
+// change), a finer cut of the last round of blocks (none), the loop over a block unrolled by two
+// (544) and four (521). The block's partial sums are formed in each warp's own shared-memory
+// area once its sweep is done, so the block needs no other shared memory.
 template <int POL>
 struct R32Shape {
     static constexpr int DEG = 6, D = 2, BS = 8;
-    static constexpr int WARPS = POL ? 8 : 7, MIN_BLOCKS = POL ? 3 : 4;
-    static constexpr int ROWS = D * (DEG + 1) * 32 * 16;
+    static constexpr int WARPS = 8, MIN_BLOCKS = 3;
+    static constexpr int ROW = kPlanarRow * 4;  // bytes
+    static constexpr int ROWS = D * (DEG + 1) * ROW;
     static constexpr int LINK_BYTES = BS * DEG * 8;
     static constexpr int POL_OFF = LINK_BYTES + BS * 4;
     static constexpr int SLOT = POL_OFF + (POL ? BS * 8 : 0);
@@ -81,10 +89,15 @@ __device__ __forceinline__ void renorm_block32(const PassArgs &a, float4 *S, int
         float4 v[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (h + k < n) v[k] = __ldcg(S + (int64_t)(g0 + h + k) * 32 + lane);
+            if (h + k < n) {
+                const float *row = (const float *)(S + (int64_t)(g0 + h + k) * 32);
+                const float2 xy = __ldcg((const float2 *)row + lane);
+                v[k] = make_float4(xy.x, xy.y, __ldcg(row + 64 + lane), 0.f);
+            }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (h + k < n) S[(int64_t)(g0 + h + k) * 32 + lane] = renorm_spin32(v[k], __ldg(a.fold_norm + g0 + h + k));
+            if (h + k < n)
+                planar_set((float *)(S + (int64_t)(g0 + h + k) * 32), lane, renorm_spin32(v[k], __ldg(a.fold_norm + g0 + h + k)));
     }
 }
 
@@ -113,27 +126,20 @@ __global__ void __launch_bounds__(R32Shape<POL>::WARPS * 32, R32Shape<POL>::MIN_
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = lane;
     unsigned char *wbase = smem + warp * WARP_BYTES;
-    float4 *rows = (float4 *)wbase;
     unsigned char *lslots = wbase + ROWS;
     float4 *S = (float4 *)a.spins;
-    const float4 *Sr = S + r;
+    // a site's rows are 7 x 24 16-byte pieces; piece k = lane + 32 i is part of row k / 24. Rows
+    // i and i + 3 of a lane are four apart and their pieces at the same place in the row.
+    const int k1 = lane + 32, k2 = lane + 64;
+    const unsigned char *src0 = (const unsigned char *)S + lane % 24 * 16, *src1 = (const unsigned char *)S + k1 % 24 * 16,
+                        *src2 = (const unsigned char *)S + k2 % 24 * 16;
+    const int row0 = lane / 24 * 8, row1 = k1 / 24 * 8, row2 = k2 / 24 * 8;  // of a link, bytes
     const int2 *E = (const int2 *)a.edges;
     const uint32_t inst = (uint32_t)(a.inst0 + r);
     const double *sc = rs_->sched + ((int64_t)step_idx * a.n_inst + a.inst_local0 + r) * 2;
     const float beta = (float)sc[0], B = (float)sc[1];
     const float sigma = (POL && rs_->sigma) ? (float)rs_->sigma[a.inst_local0 + r] : 0.f;
     const int g_end = a.g_end;
-    uint32_t rk0[10], rk1[10];
-    {
-        uint32_t x = (uint32_t)a.seed, y = (uint32_t)(a.seed >> 32);
-#pragma unroll
-        for (int q = 0; q < 10; ++q) {
-            rk0[q] = x;
-            rk1[q] = y;
-            x += 0x9E3779B9u;
-            y += 0xBB67AE85u;
-        }
-    }
     auto issue_links = [&](int sb, int slot) {
         if (sb >= g_end) return;
         const int ns = min(BS, g_end - sb);
@@ -148,17 +154,19 @@ __global__ void __launch_bounds__(R32Shape<POL>::WARPS * 32, R32Shape<POL>::MIN_
     };
     auto issue_rows = [&](int g, int lslot, int j, int rslot) {
         if (g >= g_end) return;
-        const int4 *lk = (const int4 *)(lslots + lslot * SLOT) + j * (DEG / 2);
-        float4 *dst = rows + rslot * (DEG + 1) * 32 + lane;
+        const unsigned char *lk = lslots + lslot * SLOT + j * (DEG * 8);
+        unsigned char *dst = wbase + rslot * (DEG + 1) * Sh::ROW + lane * 16;
         VEGAS_CHECK(g < a.n_sites_total, 14, g);
-#pragma unroll
-        for (int q = 0; q < DEG / 2; ++q) {
-            const int4 l = lk[q];
-            VEGAS_CHECK(l.x >= 0 && l.x < a.n_sites_total && l.z >= 0 && l.z < a.n_sites_total, 15, l.x);
-            cp16(dst + (2 * q) * 32, Sr + (int64_t)l.x * R);
-            cp16(dst + (2 * q + 1) * 32, Sr + (int64_t)l.z * R);
-        }
-        cp16(dst + DEG * 32, Sr + (int64_t)g * R);
+        const int j0 = *(const int *)(lk + row0), j1 = *(const int *)(lk + row1), j2 = *(const int *)(lk + row2);
+        const int j3 = *(const int *)(lk + row0 + 32);
+        const int j4 = lane < 16 ? *(const int *)(lk + 40) : g;
+        VEGAS_CHECK(min(min(j0, j1), min(j2, j3)) >= 0 && max(max(j0, j1), max(j2, j3)) < a.n_sites_total && j4 >= 0 && j4 < a.n_sites_total, 15, j0);
+        cp16(dst, src0 + (int64_t)j0 * (R * 16));
+        cp16(dst + 512, src1 + (int64_t)j1 * (R * 16));
+        cp16(dst + 1024, src2 + (int64_t)j2 * (R * 16));
+        cp16(dst + 1536, src0 + (int64_t)j3 * (R * 16));
+        cp16(dst + 2048, src1 + (int64_t)j4 * (R * 16));
+        if (lane < 8) cp16(dst + 2560, src2 + (int64_t)g * (R * 16));
     };
 
     const uint32_t n_blocks = (uint32_t)(g_end - a.g_begin + BS - 1) / BS;  // a ticket past them ends the warp
@@ -188,7 +196,7 @@ __global__ void __launch_bounds__(R32Shape<POL>::WARPS * 32, R32Shape<POL>::MIN_
                 const unsigned char *slot = lslots + ls * SLOT;
                 const uint32_t orig = ((const uint32_t *)(slot + LINK_BYTES))[j];
                 staged_attempt<DEG, PM, LM, POL, RN != 0>(a, (const int4 *)slot + j * (DEG / 2),
-                                                 rows + (j & 1) * (DEG + 1) * 32 + lane, orig, g, r, R, t, inst, rk0, rk1,
+                                                 PlanarRows{(const float *)(wbase + (j & 1) * (DEG + 1) * Sh::ROW), lane}, orig, g, r, R, t, inst, a.rk0, a.rk1,
                                                  beta, B, S, acc, nan_seen, log_accepts,
                                                  (const PolicySite32 *)(slot + POL_OFF) + j, sigma);
             }

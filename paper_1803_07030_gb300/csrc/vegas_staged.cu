@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 3 : 2) pass32_staged(const 
             const unsigned char *slot = lslots + pk.lslot * G.slot_bytes;
             const int li = pk.j * G.spg + my;
             const int4 *lk = (const int4 *)slot + li * (DEG / 2);
-            const float4 *row = rows + rsl * (DEG + 1) * 32 + lane;
+            const QuadRows row{rows + rsl * (DEG + 1) * 32 + lane};
             const uint32_t orig = ((const uint32_t *)(slot + G.link_bytes))[li];
             bool skip = false;
 #ifdef VEGAS_DEBUG_CHECKS
@@ -247,6 +247,8 @@ PassFn select_pass32(const PassArgs &a) {
 }
 
 int pass32_smem(const PassArgs &a) { return use_staged(a) ? staged_smem(a) : 0; }
+
+bool pass32_r32_rows(const PassArgs &a) { return use_r32(a); }
 
 bool pass32_direct(const PassArgs &a) { return !use_staged(a); }
 

@@ -44,13 +44,26 @@ __device__ __forceinline__ uint4 trial_block32(uint32_t orig, uint32_t t, uint32
     return c;
 }
 
+// Rows staged in shared memory: spin j of the lane (neighbours, then the site's own).
+struct QuadRows {  // 32 float4 per row
+    static constexpr bool PLANAR = false;
+    const float4 *p;  // row 0, the lane's
+    __device__ __forceinline__ float4 get(int j) const { return p[j * 32]; }
+};
+struct PlanarRows {  // 32 (x, y) pairs, then 32 z
+    static constexpr bool PLANAR = true;
+    const float *p;  // row 0
+    int lane;
+    __device__ __forceinline__ float4 get(int j) const { return planar_spin(p + j * kPlanarRow, lane); }
+};
+
 // One staged attempt with its random block c already drawn: links lk (int4 pairs), rows
-// row[j*32] (neighbour j) and row[DEG*32] (own) in shared memory; with POL, the site's
+// get(j) (neighbour j) and get(DEG) (own) in shared memory; with POL, the site's
 // update policy *ps too (POL 1: the policy from the entry; POL 2 + c: every site has policy
 // c). LM 3 takes the lower sums as all (lower_all) or none at run time. RN stores the spin
 // after the attempt renormalised, accepted or not (the step's last pass over the site).
-template <int DEG, int PM, int LM, int POL = 0, bool RN = false>
-__device__ __forceinline__ void staged_attempt_rw(const PassArgs &a, const int4 *lk, const float4 *row, uint32_t orig,
+template <int DEG, int PM, int LM, int POL = 0, bool RN = false, typename Rows>
+__device__ __forceinline__ void staged_attempt_rw(const PassArgs &a, const int4 *lk, const Rows row, uint32_t orig,
                                                   int g, int r, int R, uint32_t t, uint4 c, float beta, float B,
                                                   float4 *S, Acc32 &acc, bool &nan_seen, bool log_accepts,
                                                   const PolicySite32 *ps = nullptr, float sigma = 0.f,
@@ -61,14 +74,14 @@ __device__ __forceinline__ void staged_attempt_rw(const PassArgs &a, const int4 
 #pragma unroll
     for (int j = 0; j < DEG / 2; ++j) {
         const int4 q = lk[j];
-        link32(row[(2 * j) * 32], __int_as_float(q.y), LM == 2 && q.x < a.lower_end, hxy, hz, lxy, lz);
-        link32(row[(2 * j + 1) * 32], __int_as_float(q.w), LM == 2 && q.z < a.lower_end, hxy, hz, lxy, lz);
+        link32(row.get(2 * j), __int_as_float(q.y), LM == 2 && q.x < a.lower_end, hxy, hz, lxy, lz);
+        link32(row.get(2 * j + 1), __int_as_float(q.w), LM == 2 && q.z < a.lower_end, hxy, hz, lxy, lz);
     }
     if (LM == 1 || (LM == 3 && lower_all)) {
         lxy = hxy;
         lz = hz;
     }
-    const float4 Si = row[DEG * 32];
+    const float4 Si = row.get(DEG);
     float4 Sn;
     bool ok, bad;
     float e_i;
@@ -76,18 +89,22 @@ __device__ __forceinline__ void staged_attempt_rw(const PassArgs &a, const int4 
         POL ? policy_trial32<(POL >= 2 ? POL - 2 : -1)>(*ps, sigma, Si, p.sn, c) : trial_random32(c, p.sn);
     attempt32<PM, LM == 3 ? 1 : LM>(Si, hxy, hz, lxy, lz, p, beta, B, P, c.z, Sn, ok, e_i, bad);
     nan_seen |= bad;
-    if (RN)
-        S[(int64_t)g * R + r] = renorm_spin32(Sn, __ldg(a.fold_norm + g));
-    else if (ok)
+    if (Rows::PLANAR) {
+        if (RN)
+            planar_set((float *)(S + (int64_t)g * 32), r, renorm_spin32(Sn, __ldg(a.fold_norm + g)));
+        else if (ok)
+            planar_set((float *)(S + (int64_t)g * 32), r, Sn);
+    } else if (ok) {
         S[(int64_t)g * R + r] = Sn;
+    }
     if (log_accepts)
         a.alog[(int64_t)t * a.alog_stride + a.alog_base + (int64_t)r * a.n_sample_sites + orig] = ok ? 1 : 0;
     acc.add(e_i, Sn, ok);
 }
 
 // The same, drawing the random block first.
-template <int DEG, int PM, int LM, int POL = 0, bool RN = false>
-__device__ __forceinline__ void staged_attempt(const PassArgs &a, const int4 *lk, const float4 *row, uint32_t orig,
+template <int DEG, int PM, int LM, int POL = 0, bool RN = false, typename Rows>
+__device__ __forceinline__ void staged_attempt(const PassArgs &a, const int4 *lk, const Rows row, uint32_t orig,
                                                int g, int r, int R, uint32_t t, uint32_t inst, const uint32_t *rk0,
                                                const uint32_t *rk1, float beta, float B, float4 *S, Acc32 &acc,
                                                bool &nan_seen, bool log_accepts, const PolicySite32 *ps = nullptr,

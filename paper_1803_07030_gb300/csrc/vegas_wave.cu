@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 3) wave32_r32(const WaveArgs w) {
             if (g < se) {
                 const uint32_t orig = ((const uint32_t *)(slot + kWaveLinkBytes))[j];
                 const int4 *lk = (const int4 *)slot + j * (DEG / 2);
-                const float4 *row = rows + (j & 1) * (DEG + 1) * 32 + lane;
+                const QuadRows row{rows + (j & 1) * (DEG + 1) * 32 + lane};
                 // one code path for both classes (class 0: no lower links, lower sums 0)
                 staged_attempt_rw<DEG, PM, 3>(a, lk, row, orig, g, r, R, t, trial_block32(orig, t, inst, rk0, rk1), beta,
                                               B, S, acc, nan_seen, log_accepts, nullptr, 0.f, c1);
