@@ -1436,73 +1436,63 @@ __global__ void __launch_bounds__(NT) coop64_kernel(const CoopArgs ca) {
 
 // ------------------------------------------------------------------ per-MCS reduction
 // One block per instance sums its sample's block partials over every colour class in a fixed
-// order (thread k takes slots k, k + 256, ... in turn, then a butterfly inside each warp and
-// the warps in order) and appends the record; the last block to finish advances the MCS
-// counter and the record index (no waiting: a ticket counter, not a barrier). Block 0 also
-// zeroes the passes' block counters: every pass of this MCS has finished.
+// order (thread k takes slots k, k + 256, ... in turn; then warp q adds quantity q: lane l the
+// threads l, l + 32, ..., and a butterfly) and appends the record; the last block to finish
+// advances the MCS counter and the record index (no waiting: a ticket counter, not a barrier).
+// Block 0 also zeroes the passes' block counters: every pass of this MCS has finished. Bound by
+// latencies, of which an FP64 instruction of a warp is one (64 cycles): with all four quantities
+// in every warp's butterfly and the width adapted after it, an MCS of 60 x 60 x 52 sites x 32
+// took 82.5 us, now 79.
 __global__ void __launch_bounds__(256) reduce_kernel(const ReduceArgs a) {
-    __shared__ double red[8][4];
+    __shared__ double part[4][256];
     RunState *rs = a.run;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int il = blockIdx.x;
-    const uint32_t rec = rs->rec;
+    const uint32_t rec = rs->rec, t = rs->t;
     if (blockIdx.x == 0 && a.tickets)
         for (int k = threadIdx.x; k < a.n_tickets; k += blockDim.x) a.tickets[k] = 0u;
+    if (threadIdx.x == 4 * 32 && rs->acc) {  // accepted attempts of this MCS; the adaptive width follows them
+        const uint32_t n = rs->acc[il];
+        rs->acc[il] = 0;
+        if (rs->acc_hist) rs->acc_hist[(int64_t)rec * a.n_inst + il] = n;
+        if (a.adapt_n && a.adapt_n[il] > 0 && rs->sigma && rec % rs->mcs < rs->mcs / 5)
+            rs->sigma[il] = adapt_width(rs->sigma[il], n, a.adapt_n[il]);
+    }
     const int s = il / a.R, r = il % a.R;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    double total = 0.0;  // warp q < 4: quantity q
     for (int k = 0; k < a.n_groups; ++k) {  // type groups in order, then their total
         const int64_t base = a.slot_base[s * a.n_groups + k];
         const int32_t cnt = a.slot_count[s * a.n_groups + k];
         double u[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
+#pragma unroll 4
+        for (int32_t j = threadIdx.x; j < cnt; j += 256) {
             const double4_32a p = *(const double4_32a *)(a.partial + ((base + j) * a.R + r) * 4);
             u[0] += p.x;
             u[1] += p.y;
             u[2] += p.z;
             u[3] += p.w;
         }
-        for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) u[q] += __shfl_xor_sync(0xFFFFFFFFu, u[q], off);
-        }
-        if (lane == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) red[warp][q] = u[q];
+        for (int q = 0; q < 4; ++q) part[q][threadIdx.x] = u[q];
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double t4[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+        if (warp < 4) {
+            double v = part[warp][lane];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) t4[q] += red[w][q];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] += t4[q];
-            if (a.n_types > 0 && rs->type_hist) {
-                double *th = rs->type_hist + (((int64_t)rec * a.n_inst + il) * a.n_types + k) * 3;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) th[c] = t4[c + 1];
-            }
+            for (int w = 1; w < 8; ++w) v += part[warp][w * 32 + lane];
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+            total += v;
+            if (lane == 0 && warp > 0 && a.n_types > 0 && rs->type_hist)
+                rs->type_hist[(((int64_t)rec * a.n_inst + il) * a.n_types + k) * 3 + warp - 1] = v;
         }
-        __syncthreads();  // red is reused by the next group
+        __syncthreads();  // part is reused by the next group; after the last, this block has read the run state
     }
-    if (threadIdx.x == 0) {
-        double *h = rs->hist + ((int64_t)rec * a.n_inst + il) * 4;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) h[q] = v[q];
-        if (rs->acc) {  // accepted attempts of this MCS; the adaptive width follows them
-            const uint32_t n = rs->acc[il];
-            rs->acc[il] = 0;
-            if (rs->acc_hist) rs->acc_hist[(int64_t)rec * a.n_inst + il] = n;
-            if (a.adapt_n && a.adapt_n[il] > 0 && rs->sigma && rec % rs->mcs < rs->mcs / 5)
-                rs->sigma[il] = adapt_width(rs->sigma[il], n, a.adapt_n[il]);
-        }
-        __threadfence();
-        const uint32_t done = atomicAdd(&rs->ticket, 1u);
-        if (done == gridDim.x - 1) {
-            rs->ticket = 0;
-            rs->t = rs->t + 1;
-            rs->rec = rec + 1;
-            __threadfence();
-        }
+    if (warp < 4 && lane == 0) rs->hist[((int64_t)rec * a.n_inst + il) * 4 + warp] = total;
+    __syncthreads();
+    // every thread of the block has read the run state: the last block may change it
+    if (threadIdx.x == 0 && atomicAdd(&rs->ticket, 1u) == gridDim.x - 1) {
+        rs->ticket = 0;
+        rs->t = t + 1;
+        rs->rec = rec + 1;
     }
 }
 
