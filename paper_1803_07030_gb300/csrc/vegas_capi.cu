@@ -2048,10 +2048,10 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                     }
                     c->variant = best_v;
                     // The tiled form runs several times faster than any sweep timed above wherever it
-                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 29, 55; 32^3 x
+                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 27.5, 55; 32^3 x
                     // 32 replicas 12, 38; the 29k-site core/shell particle 4.9, 23; a 13k-site fcc sphere
                     // x 8 5.4, 24; 512 sites 2.1, 9), so it is not timed: the cooperative form's time stands
-                    // for it, at 4/7 (the least gain measured, 29 to 55, with the probes' noise; the fcc
+                    // for it, at 4/7 (the least gain measured, 29 to 55 at first, with the probes' noise; the fcc
                     // spheres: 15.6 us in clusters beside 24 and 5.4). It takes over where it adds the
                     // attempts' FP32 shares in the order of the sweep that would run (one thread per
                     // site of a class: the cooperative form, and every sweep of classes of at most 512

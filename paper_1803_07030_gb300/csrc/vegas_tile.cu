@@ -17,7 +17,7 @@
 //
 // us per MCS, before (grid barriers, neighbours in L2) and now: 64^3 with uniaxial anisotropy
 // 17.5 and 4.9, the 29k-site core/shell particle 23.0 and 4.9, a 13k-site fcc sphere x 8 replicas
-// 23.5 and 5.3, 128^3 54.6 and 29.1.
+// 23.5 and 5.3, 128^3 54.6 and 27.5.
 //
 // Why one mailbox word per site is enough: tag t + 1 marks the value after MCS t. Site i of part
 // N (class c) is read by part b because some site j of b (class c') links to i; then N reads j.
@@ -79,7 +79,10 @@ __device__ __forceinline__ void two_sum(float2 &s, float2 x, float2 &lo) {
 // keeps in shared memory beside the spins: 2 rows, site ids and remote words' indices, 1 the ids
 // and indices, 0 nothing (the rest is read through L1 from tables in the block's own order). FMT 1
 // halves the rows (samples of at most kTileCodes exchange values): for parts whose rows do not fit
-// otherwise, or are read from L2 (128^3, 100 MB of pairs: 46.8 us per MCS, 29.1 with words).
+// otherwise, or are read from L2 (128^3, 100 MB of pairs: 46.8 us per MCS, 29.1 with words; 27.5 since
+// the warps add their sums, which leaves room for 512 threads in place of 384. There it is bound by
+// the warps that fit beside 12 bytes per spin: issue 45%. Slower: rows fetched a round ahead 30.9, two
+// sites in flight per thread 30.5; rows by link pair the same).
 template <int W, int POL, int PM, int MEM, int FMT>
 __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(const TileArgs ta) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -101,6 +104,9 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
     float *s_part = (float *)(smem + ta.part_off);
     uint32_t *s_cnt = (uint32_t *)(s_part + (1 + ta.two_buffers) * 4 * NT);
     float *s_lo = (float *)(s_cnt + (1 + ta.two_buffers) * NT);
+    // MEM 0: the warps' sums, [4][NT / 32] in FP64 and [NT / 32] counts
+    double *s_sum = (double *)(smem + ta.part_off);
+    uint32_t *s_num = (uint32_t *)(s_sum + 4 * (NT >> 5));
     __shared__ int s_ok;  // 0: the record warp leaves
     RunState *rs = a.run;
     const uint32_t t0 = rs->t, rec0 = rs->rec;
@@ -132,13 +138,20 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
             const int b = m & ta.two_buffers;
             bar_sync(kBarFull + b, NT + kTileRecord);
             if (s_ok == 0) return;
-            const float *x = s_part + (b * 4 + q) * NT;
             double v = 0.0;
-            for (int k = lane; k < NT; k += 32) v += (double)x[k];
-            if (ta.long_runs && lane < (NT >> 5)) v += (double)s_lo[(b * 4 + q) * (NT >> 5) + lane];
             uint32_t n = 0;
-            if (q == 0)
-                for (int k = lane; k < NT; k += 32) n += s_cnt[b * NT + k];
+            if (MEM == 0) {
+                if (lane < (NT >> 5)) {
+                    v = s_sum[q * (NT >> 5) + lane];
+                    if (q == 0) n = s_num[lane];
+                }
+            } else {
+                const float *x = s_part + (b * 4 + q) * NT;
+                for (int k = lane; k < NT; k += 32) v += (double)x[k];
+                if (ta.long_runs && lane < (NT >> 5)) v += (double)s_lo[(b * 4 + q) * (NT >> 5) + lane];
+                if (q == 0)
+                    for (int k = lane; k < NT; k += 32) n += s_cnt[b * NT + k];
+            }
             bar_arrive(kBarEmpty + b, NT + kTileRecord);
             for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
             const int64_t at = ((int64_t)m << a.log2R) + r;
@@ -270,6 +283,31 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
         }
         // this MCS's sums of every thread (at most 64 attempts each) to the record warp
         const int b = m & ta.two_buffers;
+        if (MEM == 0) {
+            // long parts: shared memory goes to spins, so each warp adds its threads' sums, in FP64; the
+            // first two steps halve the quantities per lane (six additions for the four)
+            const int lane = tid & 31;
+            double v[4] = {(double)fem.x, (double)fxy.x, (double)fxy.y, (double)fem.y};
+            if (ta.long_runs) {
+                v[0] += (double)fem_lo.x;
+                v[1] += (double)fxy_lo.x;
+                v[2] += (double)fxy_lo.y;
+                v[3] += (double)fem_lo.y;
+            }
+            const bool hi = lane & 16, odd = lane & 8;
+            double x = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xFFFFFFFFu, hi ? v[0] : v[2], 16);
+            double y = (hi ? v[3] : v[1]) + __shfl_xor_sync(0xFFFFFFFFu, hi ? v[1] : v[3], 16);
+            x = (odd ? y : x) + __shfl_xor_sync(0xFFFFFFFFu, odd ? x : y, 8);
+            for (int off = 4; off > 0; off >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, off);
+            const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, nacc);
+            if (m > 0) bar_sync(kBarEmpty, NT + kTileRecord);
+            if ((lane & 7) == 0) s_sum[(lane >> 3) * (NT >> 5) + (tid >> 5)] = x;
+            if (lane == 0) s_num[tid >> 5] = n;
+            bar_arrive(kBarFull, NT + kTileRecord);
+            fem = fxy = fem_lo = fxy_lo = make_float2(0.f, 0.f);
+            nacc = 0;
+            continue;
+        }
         if (m > ta.two_buffers) bar_sync(kBarEmpty + b, NT + kTileRecord);
         float *o = s_part + b * 4 * NT + tid;
         o[0] = fem.x;
@@ -580,6 +618,7 @@ size_t tile_layout(TileArgs &a, const TilePlan &p, int threads) {
     a.cls_off = (int32_t)at;
     at = align(at + (size_t)a.n_colours * sizeof(TileClass));
     a.part_off = (int32_t)at;
+    if (a.mem == 0) return at + (size_t)(threads / 32) * (4 * sizeof(double) + sizeof(uint32_t));
     return at + (size_t)(1 + a.two_buffers) * (threads * 5 + threads / 32 * 4) * sizeof(float);
 }
 

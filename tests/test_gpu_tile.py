@@ -43,6 +43,7 @@ CASES = {
     "words_through_l1": (lambda: sc_periodic((60, 60, 60), bimodal_seed=2), 8, {}),
     "pairs_through_l1": (lambda: fcc_sphere(20.0, a=4.0 ** (1.0 / 3.0)).with_policy([3], [0.4]), 16, {}),
     "one_buffer": (lambda: sc_periodic((128, 128, 126), bimodal_seed=2), 1, {}),
+    "one_buffer_small_sample": (lambda: sc_periodic(30, bimodal_seed=2), 1, {"max_blocks": 2}),
 }
 
 
