@@ -705,28 +705,38 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     }
     cudaGetLastError();
     if (c->tile_threads == 0) return VEGAS_OK;
-    auto up = [&](auto *&p, const void *src, size_t bytes) {
-        void *d = nullptr;
-        const cudaError_t e = dalloc(c, &d, std::max<size_t>(bytes, 16));
-        if (e != cudaSuccess) return e;
-        c->tile_bufs.push_back(d);
-        p = (std::remove_reference_t<decltype(p)>)d;
-        return src && bytes > 0 ? cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, c->stream) : cudaSuccess;
+    // one allocation for the tables and the scratch (a dozen of them took 0.2 ms)
+    struct Table {
+        void **at;
+        const void *src;  // NULL: scratch
+        size_t bytes;
     };
+    std::vector<Table> tables;
+    auto up = [&](auto *&p, const void *src, size_t bytes) { tables.push_back({(void **)&p, src, bytes}); };
     const size_t words = (size_t)kTileMcs * c->R * ts.parts;
-    CK(c, up(a.parts, plan.parts.data(), plan.parts.size() * sizeof(TilePart)));
-    CK(c, up(a.classes, plan.classes.data(), plan.classes.size() * sizeof(TileClass)));
-    CK(c, up(a.site, plan.site.data(), plan.site.size() * sizeof(int32_t)));
-    CK(c, up(a.orig, plan.orig.data(), plan.orig.size() * sizeof(int32_t)));
-    CK(c, up(a.halo_slot, plan.halo_slot.data(), plan.halo_slot.size() * sizeof(int32_t)));
-    CK(c, up(a.pub, plan.pub.data(), plan.pub.size() * sizeof(int32_t)));
-    CK(c, up(a.rows, plan.rows.get(), plan.row_bytes));
-    CK(c, up(a.codes, plan.codes.data(), plan.codes.size() * sizeof(float)));
-    CK(c, up(a.mail, nullptr, (size_t)plan.n_mail * c->R * sizeof(float4) * (p64 ? 2 : 1)));
-    if (p64) CK(c, up(c->tile64.J, J64.data(), J64.size() * sizeof(double)));
-    CK(c, up(a.partial, nullptr, words * 4 * sizeof(double)));
-    CK(c, up(a.count, nullptr, words * sizeof(uint32_t)));
-    CK(c, up(a.abort, nullptr, sizeof(uint32_t)));
+    up(a.parts, plan.parts.data(), plan.parts.size() * sizeof(TilePart));
+    up(a.classes, plan.classes.data(), plan.classes.size() * sizeof(TileClass));
+    up(a.site, plan.site.data(), plan.site.size() * sizeof(int32_t));
+    up(a.orig, plan.orig.data(), plan.orig.size() * sizeof(int32_t));
+    up(a.halo_slot, plan.halo_slot.data(), plan.halo_slot.size() * sizeof(int32_t));
+    up(a.pub, plan.pub.data(), plan.pub.size() * sizeof(int32_t));
+    up(a.rows, plan.rows.get(), plan.row_bytes);
+    up(a.codes, plan.codes.data(), plan.codes.size() * sizeof(float));
+    up(a.mail, nullptr, (size_t)plan.n_mail * c->R * sizeof(float4) * (p64 ? 2 : 1));
+    if (p64) up(c->tile64.J, J64.data(), J64.size() * sizeof(double));
+    up(a.partial, nullptr, words * 4 * sizeof(double));
+    up(a.count, nullptr, words * sizeof(uint32_t));
+    up(a.abort, nullptr, sizeof(uint32_t));
+    size_t total = 0;
+    for (const Table &t : tables) total += (std::max<size_t>(t.bytes, 16) + 255) / 256 * 256;
+    unsigned char *mem = nullptr;
+    CK(c, dalloc(c, &mem, total));
+    c->tile_bufs.push_back(mem);
+    for (const Table &t : tables) {
+        *t.at = mem;
+        if (t.src && t.bytes > 0) CK(c, cudaMemcpyAsync(mem, t.src, t.bytes, cudaMemcpyHostToDevice, c->stream));
+        mem += (std::max<size_t>(t.bytes, 16) + 255) / 256 * 256;
+    }
     CK(c, cudaStreamSynchronize(c->stream));  // the plan goes out of scope
     c->tile64.t = a;
     c->tile_ok = true;
