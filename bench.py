@@ -829,7 +829,7 @@ def run_ising(args):
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "G warp-instructions/s",
                      "frac": None if achieved is None else achieved / peak,
                      "peak_source": "152 SMs x 4 issue slots x median SM clock (derived)",
-                     "kernel": "ising_pass_kernel<2>", "warp_instructions_per_attempt": inst,
+                     "kernel": "ising_pass_kernel<2, 2, 1>", "warp_instructions_per_attempt": inst,
                      "attempts_per_launch": per_launch, "avg_launch_ms": launch_ms},
         "cpu_baseline": {"value": 256 * 256 * 4 * 10 / cpu_dt, "unit": "attempts/s", "cores": 1, "kind": "oracle", "host": host_description(),
                          "sample": "256^2 x 4 replicas x 10 MCS"},

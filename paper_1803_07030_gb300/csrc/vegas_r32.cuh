@@ -27,9 +27,9 @@ namespace {
 // alone compiled in (each site's parameter still comes from its entry).
 // Rows are kept in planes (384 bytes of a site's 512): what the kernel moves most. A site's seven
 // rows come as 168 16-byte pieces, lane + 32 i the i-th of a lane. Per launch on 128^3 sites x 32,
-// against rows of 32 float4: 1.23 GB of DRAM traffic against 1.48, 217 M warp instructions
-// against 211, issue 70% against 61, 254 us against 274; on 256^3 1.95 ms against 2.04. It is now
-// bound by issue and the shared-memory pipe (61%) more than by DRAM (61%). The Philox round keys
+// against rows of 32 float4: 1.21 GB of DRAM traffic against 1.48, 208 M warp instructions
+// against 212, issue 66% against 62, 255 us against 282 (under ncu); on 256^3 1.90 ms against 2.04.
+// Issue, the shared-memory pipe (61%) and DRAM (60%) are now about equally busy. The Philox round keys
 // are kernel arguments, which frees 20 registers; yet 24 warps per SM (8 x 3) stay the best:
 // 513 us per MCS on 128^3, 28 warps 522, 32 warps 544, 36 warps 567, 16 warps 567. Also tried:
 // alternate directions of the passes, so that one starts where the other ended in L2 (no
