@@ -1354,8 +1354,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
                         const float J = in ? (float)l.J[(size_t)(e0 + w)] : 0.0f;
                         const uint32_t link = (uint32_t)j | (in && j < l.cstart[(size_t)q] ? 0x10000u : 0u);
                         if (words) {
-                            if (h_codes[code] != J)
-                                for (code = 0; h_codes[code] != J; ++code) {}
+                            code = exchange_code(h_codes, J, code);
                             row[w] = link | code << 17;
                         } else {
                             row[2 * w] = link;

@@ -30,6 +30,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
@@ -535,8 +536,13 @@ void exchange_values(const double *J, int64_t n_links, std::vector<float> &value
         if (to.size() <= (size_t)kTileCodes && std::find(to.begin(), to.end(), v) == to.end()) to.push_back(v);
     };
     auto scan = [&](std::vector<float> &to, int64_t e0, int64_t e1) {
+        double a = NAN, b = NAN;  // two values seen: a glass has two, in random order
         for (int64_t e = e0; e < e1; ++e)
-            if (e == e0 || J[e] != J[e - 1]) add(to, (float)J[e]);
+            if ((J[e] != a) & (J[e] != b)) {
+                add(to, (float)J[e]);
+                b = a;
+                a = J[e];
+            }
     };
     const int32_t chunks = (int32_t)std::min<int64_t>(16, n_links / (1 << 19) + 1);  // a thread costs 0.05 ms
     std::vector<std::vector<float>> got((size_t)chunks);
@@ -587,8 +593,7 @@ void write_tables(const TileArgs &a, const TileShape &s, TilePlan &p) {
                     J = (float)s.J[e0 + w];
                 }
                 if (a.n_codes) {
-                    if (p.codes[code] != J)
-                        for (code = 0; p.codes[code] != J; ++code) {}
+                    code = exchange_code(p.codes, J, code);
                     ((uint32_t *)p.rows.get())[at + w] = link | code << 17;
                 } else {
                     int2 x = make_int2((int)link, 0);
