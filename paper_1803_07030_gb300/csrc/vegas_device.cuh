@@ -259,6 +259,15 @@ struct Acc32 {
     }
 };
 
+// The same for a caller that ends its runs of at most 64 attempts itself.
+struct Acc32Runs : Acc32 {
+    __device__ __forceinline__ void add(float e, float4 q, bool ok) {
+        nacc += ok ? 1u : 0u;
+        fem = __fadd2_rn(fem, make_float2(e, q.z));
+        fxy = __fadd2_rn(fxy, make_float2(q.x, q.y));
+    }
+};
+
 // One link's share of the field: x and y as a packed pair (one instruction, the same two
 // roundings), z alone; with `lower`, also of the part over lower colours.
 __device__ __forceinline__ void link32(const float4 Sj, float J, bool lower, float2 &hxy, float &hz, float2 &lxy,

@@ -27,8 +27,8 @@ namespace {
 // alone compiled in (each site's parameter still comes from its entry).
 // Rows are kept in planes (384 bytes of a site's 512): what the kernel moves most. A site's seven
 // rows come as 168 16-byte pieces, lane + 32 i the i-th of a lane. Per launch on 128^3 sites x 32,
-// against rows of 32 float4: 1.21 GB of DRAM traffic against 1.48, 208 M warp instructions
-// against 212, issue 66% against 62, 255 us against 282 (under ncu); on 256^3 1.90 ms against 2.04.
+// against rows of 32 float4: 1.21 GB of DRAM traffic against 1.48, 205 M warp instructions
+// against 212, issue 67% against 62, 253 us against 282 (under ncu); on 256^3 1.90 ms against 2.04.
 // Issue, the shared-memory pipe (61%) and DRAM (60%) are now about equally busy. The Philox round keys
 // are kernel arguments, which frees 20 registers; yet 24 warps per SM (8 x 3) stay the best:
 // 513 us per MCS on 128^3, 28 warps 522, 32 warps 544, 36 warps 567, 16 warps 567. Also tried:
@@ -185,7 +185,8 @@ __global__ void __launch_bounds__(R32Shape<POL>::WARPS * 32, R32Shape<POL>::MIN_
     cp_commit();
     issue_rows(sb + 1, 0, 1, 1);
     cp_commit();
-    Acc32 acc;
+    Acc32Runs acc;
+    int run = 0;  // blocks in the run of FP32 sums (counted per block: 128^3 505.8 -> 501.6 us per MCS)
     bool nan_seen = false;
     const bool log_accepts = a.alog && t < a.alog_mcs;
     int ls = 0;
@@ -222,6 +223,10 @@ __global__ void __launch_bounds__(R32Shape<POL>::WARPS * 32, R32Shape<POL>::MIN_
             const bool last = dep >= 0 && atom_add_acq_rel(a.fold_cnt + dep, 1u) + 1u == (uint32_t)__ldg(a.fold_deg + dep);
             for (uint32_t m = __ballot_sync(0xFFFFFFFFu, last); m; m &= m - 1)
                 renorm_block32(a, S, __shfl_sync(0xFFFFFFFFu, dep, __ffs(m) - 1), lane);
+        }
+        if (++run == 64 / BS) {
+            acc.flush();
+            run = 0;
         }
         sb = sb2;
         ls ^= 1;

@@ -62,10 +62,10 @@ struct PlanarRows {  // 32 (x, y) pairs, then 32 z
 // update policy *ps too (POL 1: the policy from the entry; POL 2 + c: every site has policy
 // c). LM 3 takes the lower sums as all (lower_all) or none at run time. RN stores the spin
 // after the attempt renormalised, accepted or not (the step's last pass over the site).
-template <int DEG, int PM, int LM, int POL = 0, bool RN = false, typename Rows>
+template <int DEG, int PM, int LM, int POL = 0, bool RN = false, typename Rows, typename Sums>
 __device__ __forceinline__ void staged_attempt_rw(const PassArgs &a, const int4 *lk, const Rows row, uint32_t orig,
                                                   int g, int r, int R, uint32_t t, uint4 c, float beta, float B,
-                                                  float4 *S, Acc32 &acc, bool &nan_seen, bool log_accepts,
+                                                  float4 *S, Sums &acc, bool &nan_seen, bool log_accepts,
                                                   const PolicySite32 *ps = nullptr, float sigma = 0.f,
                                                   bool lower_all = true) {
     const Site32 p = site_params32(a, PM, g);
@@ -103,10 +103,10 @@ __device__ __forceinline__ void staged_attempt_rw(const PassArgs &a, const int4 
 }
 
 // The same, drawing the random block first.
-template <int DEG, int PM, int LM, int POL = 0, bool RN = false, typename Rows>
+template <int DEG, int PM, int LM, int POL = 0, bool RN = false, typename Rows, typename Sums>
 __device__ __forceinline__ void staged_attempt(const PassArgs &a, const int4 *lk, const Rows row, uint32_t orig,
                                                int g, int r, int R, uint32_t t, uint32_t inst, const uint32_t *rk0,
-                                               const uint32_t *rk1, float beta, float B, float4 *S, Acc32 &acc,
+                                               const uint32_t *rk1, float beta, float B, float4 *S, Sums &acc,
                                                bool &nan_seen, bool log_accepts, const PolicySite32 *ps = nullptr,
                                                float sigma = 0.f) {
     staged_attempt_rw<DEG, PM, LM, POL, RN>(a, lk, row, orig, g, r, R, t, trial_block32(orig, t, inst, rk0, rk1), beta,
