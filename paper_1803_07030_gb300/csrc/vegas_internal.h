@@ -399,9 +399,9 @@ void launch_snapshot(const void *spins, void *snap, int64_t n16, const RunState 
 constexpr int kOnceThreads = 256;  // most threads per block
 constexpr int kOnceBlocks = 8;     // most blocks (the portable cluster size)
 // Most attempts of a class, four rounds of the cluster: a round of the two classes of a simple
-// cubic sample takes 3 us, one launch per class 26 us more than the one launch. Calls from
-// Python, one launch and one per class: 27 and 54 us up to 1000 sites, 39 and 56 at 8192
-// attempts per class, 52 and 56 at 16384, 108 and 62 at 55296.
+// cubic sample takes 3 us, the launches of the other path 16 us more than the one launch. Calls
+// from Python, one launch and one per class: 27 and about 43 us up to 1000 sites, 39 and 43 at 8192
+// attempts per class, 52 and 44 at 16384.
 constexpr int64_t kOnceWork = 4 * kOnceThreads * kOnceBlocks;
 
 struct OnceArgs {

@@ -70,8 +70,9 @@ def test_one_launch_equals_a_launch_per_class(torch, case):
     assert np.abs(sums_all / many - sums).max() <= 1e-12 * max(1.0, np.abs(sums).max())
 
 
-def test_nan_is_reported(torch):
-    s = sc_periodic(4)
+@pytest.mark.parametrize("side", [4, 30])  # one launch; a launch per class
+def test_nan_is_reported(torch, side):
+    s = sc_periodic(side)
     good = np.tile([0.0, 0.0, 1.0], (s.n_sites, 1))
     for bad in (False, True, False):
         if bad:
