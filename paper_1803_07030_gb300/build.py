@@ -17,7 +17,7 @@ LIB = os.path.join(OUT_DIR, "libvegas.so")
 LIB_DEBUG = os.path.join(OUT_DIR, "libvegas_debug.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["vegas_kernels.cu", "vegas_staged.cu", "vegas_policy32.cu", "vegas_r32_renorm.cu", "vegas_wave.cu", "vegas_tile.cu", "vegas_tile64.cu", "vegas_batch.cu", "vegas_analysis.cu", "vegas_ising.cu", "vegas_capi.cu", "vegas_noalloc.cu", "vegas_loader.cpp"]
-HEADERS = ["vegas_internal.h", "vegas_device.cuh", "vegas_staged.cuh", "vegas_r32.cuh", "vegas_tile.h", "vegas_tile.cuh", "vegas_fp64.cuh", "vegas_exp64.cuh", os.path.join("..", "..", "include", "vegas.h")]
+HEADERS = ["vegas_internal.h", "vegas_device.cuh", "vegas_staged.cuh", "vegas_r32.cuh", "vegas_tile.h", "vegas_order.h", "vegas_tile.cuh", "vegas_fp64.cuh", "vegas_exp64.cuh", os.path.join("..", "..", "include", "vegas.h")]
 
 
 def _nvcc() -> str:

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "vegas_internal.h"
+#include "vegas_order.h"
 #include "vegas_tile.h"
 
 using namespace vegas;
@@ -128,6 +129,7 @@ struct vegas_ctx {
     bool res_smem = false;           // the resident sweep keeps spins in shared memory
     bool cluster_smem = false;       // the cluster sweep keeps copies of the spins in shared memory
     bool batch_ok = false;           // both run as batch32_kernel (uniform trials, no per-type sums)
+    bool probing = false;            // the autotuner times the sweeps: the former kernels run
     BatchArgs batch{};               // its tables
     int res_items = 0;          // instances of the resident and cluster sweeps
     bool res_policy = false;    // some sample has a policy table (kernel choice for the shapes)
@@ -139,7 +141,6 @@ struct vegas_ctx {
     int cluster_cs = 0, cluster_n = 0, cluster_threads = 256;
     // cooperative sweep
     bool coop_eligible = false;
-    int32_t max_class_sites = 0;  // one sample: its widest colour class
     CoopArgs coop{};
     int coop_grid = 1;
     int coop_grid_max = 1;  // every block the GPU holds at once, capped by the widest class and max_blocks
@@ -149,6 +150,7 @@ struct vegas_ctx {
     // shared memory); the grid-barrier form serves the others
     bool tile_ok = false;
     bool use_tile = false;  // the cooperative sweep runs it (not while the autotuner times the sweeps)
+    TileOrder tile_order{};  // FP32
     TileArgs tile{};
     Tile64Args tile64{};  // its FP64 counterpart (uniform trials)
     int tile_threads = 0;
@@ -278,9 +280,11 @@ int ilog2(int v) {
 // the spins in global memory, when that form does not fit the device.
 constexpr int64_t kResSmemBytes = 200 * 1024;  // spins in shared memory: 12 bytes per site
 
-// The shared-memory forms run as batch32_kernel (blocks of 512 threads, groups of at least 128).
+// The shared-memory forms run as batch32_kernel (blocks of 512 threads, groups of at least 128). Not while
+// the autotuner times them: the shape decides which sites a thread adds in FP32, so it stays the one
+// that resident32_kernel and cluster32_kernel are fastest with.
 bool batch_form(const vegas_ctx *c, int threads, int group_threads) {
-    return c->batch_ok && threads == kBatchThreads && (group_threads == 0 || group_threads >= 128);
+    return c->batch_ok && !c->probing && threads == kBatchThreads && (group_threads == 0 || group_threads >= 128);
 }
 
 bool set_resident_shape(vegas_ctx *c, int threads, int group_threads = 0, int group_sites = 0, bool smem = false) {
@@ -446,6 +450,17 @@ void enqueue_cluster(vegas_ctx *c, cudaStream_t st, int32_t n) {
         launch_cluster(a, c->cluster_n, c->cluster_cs, c->cluster_threads, st);
     }
     launch_advance(c->d_run, n, st);
+}
+
+// Whether the tiled sweep may take the place of sweep v in its present shape (FP64: every sweep
+// records the same sums to their rounding).
+bool tile_for(const vegas_ctx *c, int v) {
+    if (!c->tile_ok) return false;
+    if (c->precision == 64) return true;
+    const int64_t at_once = v == 1   ? c->res_threads
+                            : v == 2 ? ((int64_t)c->coop_grid * kCoopThreads) >> c->log2R
+                                     : (int64_t)c->cluster_cs * c->cluster_threads;
+    return tile_in_order(c->tile_order, v, at_once);
 }
 
 // One MCS of the wavefront sweep (both colour classes in one launch), then the reduction;
@@ -659,7 +674,6 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     for (int32_t g = 0; g < si.n; ++g) max_deg = std::max(max_deg, l.row_ptr[(size_t)g + 1] - l.row_ptr[(size_t)g]);
     int32_t widest = 1;
     for (int32_t q = 0; q < si.n_colours; ++q) widest = std::max(widest, si.cstart[(size_t)q + 1] - si.cstart[(size_t)q]);
-    c->max_class_sites = widest;
     const int blocks = o.max_blocks > 0 ? std::min(c->sm_count, o.max_blocks) : c->sm_count;
     TileShape ts{};
     ts.n = si.n;
@@ -739,6 +753,7 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     }
     CK(c, cudaStreamSynchronize(c->stream));  // the plan goes out of scope
     c->tile64.t = a;
+    c->tile_order = TileOrder{plan.columns, widest, si.n, c->R, plan.run};
     c->tile_ok = true;
     return VEGAS_OK;
 }
@@ -1384,12 +1399,15 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
             ba.codes = c->d_batch_codes;
             ba.modes = c->d_batch_modes;
         }
-        // the forms with policies or per-type sums, and blocks of 256 or groups of 64 threads when asked for
-        if (c->res_smem_eligible && (!c->batch_ok || o.group_threads == 64 || o.resident_smem == 1)) {
+        // the forms with policies or per-type sums, blocks of 256 or groups of 64 threads when asked for, and
+        // the autotuner's timings
+        if (c->res_smem_eligible) {
             h_ell.assign((size_t)n_sites * kEllRow, make_int2(-1, 0));
-            for (int64_t g = 0; g < n_sites; ++g)
-                for (int64_t e = h_rowptr[(size_t)g]; e < h_rowptr[(size_t)g + 1]; ++e)
-                    h_ell[(size_t)g * kEllRow + (size_t)(e - h_rowptr[(size_t)g])] = h_e32[(size_t)e];
+            host_ranges(n_sites, (int32_t)std::min<int64_t>(16, n_sites / 32768 + 1), [&](int64_t g0, int64_t g1) {
+                for (int64_t g = g0; g < g1; ++g)
+                    for (int64_t e = h_rowptr[(size_t)g]; e < h_rowptr[(size_t)g + 1]; ++e)
+                        h_ell[(size_t)g * kEllRow + (size_t)(e - h_rowptr[(size_t)g])] = h_e32[(size_t)e];
+            });
             DALLOC(c->d_ell, sizeof(int2) * h_ell.size());
             H2D(c->d_ell, h_ell.data(), sizeof(int2) * h_ell.size());
         }
@@ -1679,7 +1697,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
             return bail(VEGAS_EINVAL);
         }
         c->variant = 2;
-        c->use_tile = c->tile_ok;
+        c->use_tile = tile_for(c, 2);
         c->tuned = true;
     } else if (o.variant == 3) {
         if (!c->cluster_eligible) {
@@ -1791,6 +1809,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             }
         if ((st = set_device(c)) != VEGAS_OK) return st;
         NvtxRange run_range("vegas_run");
+        c->probing = false;  // a timing that an error ended
         const int64_t nrec = (int64_t)n_steps * mcs;
         if (sched.size() > c->sched_cap) {
             if (c->d_sched) {
@@ -2024,6 +2043,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                     int best_v = c->variant;
                     Cand best_c = cand[0];
                     const int cs_rule = c->cluster_cs, ct_rule = c->cluster_threads, rt_rule = c->res_threads;
+                    c->probing = true;
                     for (const Cand &vc : cand) {
                         const int v = vc.v;
                         // grouped instances: group_threads threads for up to 16 sites each per thread
@@ -2045,6 +2065,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                         cudaEventDestroy(x1);
                         if (c->tune_ms[v] == 0.0 || ms / probe < c->tune_ms[v]) c->tune_ms[v] = ms / probe;
                         sweep_ms += ms;
+                        if (v == 0) ms = (float)(1e-3 * probe * per_class_us(1e3 * ms / probe, c->n_planar > 0));
                         if (v == cand[0].v || ms < best) {
                             best = ms;
                             best_v = v;
@@ -2056,26 +2077,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                         if (e4) break;  // report the device error below
                     }
                     c->variant = best_v;
-                    // The tiled form runs several times faster than any sweep timed above wherever it
-                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 27.5, 55; 32^3 x
-                    // 32 replicas 12, 38; the 29k-site core/shell particle 4.9, 23; a 13k-site fcc sphere
-                    // x 8 5.4, 24; 512 sites 2.1, 9), so it is not timed: the cooperative form's time stands
-                    // for it, at 4/7 (the least gain measured, 29 to 55 at first, with the probes' noise; the fcc
-                    // spheres: 15.6 us in clusters beside 24 and 5.4). It takes over where it adds the
-                    // attempts' FP32 shares in the order of the sweep that would run (one thread per
-                    // site of a class: the cooperative form, and every sweep of classes of at most 512
-                    // sites) or where that order is not fixed anyway (the kernel of 32 replicas draws its
-                    // blocks from a counter); elsewhere records would differ by the FP32 sums' rounding,
-                    // 1e-9 of their norm.
-                    if (c->tile_ok && !c->opt.resident_smem &&
-                        (best_v == 2 ||
-                         (c->tune_ms[2] > 0.0 && c->tune_ms[2] * probe <= 1.75 * best) ||
-                         c->max_class_sites <= kTileThreads ||
-                         (best_v == 0 && pass32_kind(c->passes[0].args) == VEGAS_KERNEL_PASS32_R32))) {
-                        c->variant = best_v = 2;
-                        best_c = Cand{2, 2, 0, 0, 0};
-                        c->use_tile = true;
-                    }
+                    c->probing = false;
                     // the shape of the sweep kept goes last: the two persistent sweeps share the
                     // grouping of small instances
                     if (c->cluster_eligible && best_v != 3) set_cluster_shape(c, cs_rule, ct_rule, 0, 0, 0);
@@ -2087,6 +2089,15 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                     if (best_v == 3)
                         set_cluster_shape(c, best_c.a, best_c.b, best_c.split, best_c.group, best_c.group * 16,
                                           best_c.sm != 0);
+                    // The tiled form runs several times faster than the sweeps timed above wherever it
+                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 27.5, 55; the
+                    // 29k-site core/shell particle 4.9, 23; a 13k-site fcc sphere x 8 5.4, 24; 512 sites 2.1, 9),
+                    // so it is not timed: it takes the place of the one kept where it records what that
+                    // one would.
+                    if (!c->opt.resident_smem && tile_for(c, best_v)) {
+                        c->variant = 2;
+                        c->use_tile = true;
+                    }
                 }
                 c->tuned = true;
             }

@@ -64,16 +64,6 @@ struct TilePrep {
     TileRow<W, FMT> row;
 };
 
-// s += x in FP32 (both lanes), the exact rounding errors of the two additions added to lo (Knuth's
-// TwoSum).
-__device__ __forceinline__ void two_sum(float2 &s, float2 x, float2 &lo) {
-    const float2 t = __fadd2_rn(s, x), b = __fadd2_rn(t, make_float2(-s.x, -s.y));
-    const float2 a = __fadd2_rn(t, make_float2(-b.x, -b.y));
-    const float2 e = __fadd2_rn(__fadd2_rn(s, make_float2(-a.x, -a.y)), __fadd2_rn(x, make_float2(-b.x, -b.y)));
-    lo = __fadd2_rn(lo, e);
-    s = t;
-}
-
 // W: links per fixed row (6 or kEllRow; shorter rows are padded with links of J = 0 to the site
 // itself, which add signed zeros). PM: 0 uniform parameters without anisotropy, 3 no cubic
 // anisotropy, 2 any. MEM: what a block
@@ -101,10 +91,9 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
     int32_t *s_pub = (int32_t *)(smem + ta.pub_off);
     int32_t *s_slot = (int32_t *)(smem + ta.slot_off);
     TileClass *s_cls = (TileClass *)(smem + ta.cls_off);
-    // one or two buffers of [E, Mx, My, Mz][NT], of [NT] counts, and of [4][NT / 32] rounding errors
+    // one or two buffers of [E, Mx, My, Mz][NT], and of [NT] counts
     float *s_part = (float *)(smem + ta.part_off);
     uint32_t *s_cnt = (uint32_t *)(s_part + (1 + ta.two_buffers) * 4 * NT);
-    float *s_lo = (float *)(s_cnt + (1 + ta.two_buffers) * NT);
     // MEM 0: the warps' sums, [4][NT / 32] in FP64 and [NT / 32] counts
     double *s_sum = (double *)(smem + ta.part_off);
     uint32_t *s_num = (uint32_t *)(s_sum + 4 * (NT >> 5));
@@ -149,7 +138,6 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
             } else {
                 const float *x = s_part + (b * 4 + q) * NT;
                 for (int k = lane; k < NT; k += 32) v += (double)x[k];
-                if (ta.long_runs && lane < (NT >> 5)) v += (double)s_lo[(b * 4 + q) * (NT >> 5) + lane];
                 if (q == 0)
                     for (int k = lane; k < NT; k += 32) n += s_cnt[b * NT + k];
             }
@@ -190,9 +178,8 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
         q.P = POL ? policy_trial32(a.pol32[g], 0.f, q.Si, q.p.sn, rw) : trial_random32(rw, q.p.sn);
         q.wacc = rw.z;
     };
-    // the thread's sums of E and Mz, Mx and My over the MCS: one attempt per class, or with long_runs
-    // several, whose rounding errors are then summed beside them
-    float2 fem = make_float2(0.f, 0.f), fxy = fem, fem_lo = fem, fxy_lo = fem;
+    // the thread's sums of E and Mz, Mx and My over the MCS
+    float2 fem = make_float2(0.f, 0.f), fxy = fem;
     uint32_t nacc = 0;
     auto finish = [&](int k, uint32_t t, const TilePrep<W, FMT> &q, const TileClass &cl) {
         // the field in row order (l: its part over lower colours)
@@ -219,14 +206,8 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
         if (ok) loc_set(sp, cap, k, Sn.x, Sn.y, Sn.z);
         nan_seen |= bad;
         nacc += ok ? 1u : 0u;
-        const float2 ez = make_float2(e, Sn.z), xy = make_float2(Sn.x, Sn.y);
-        if (ta.long_runs) {
-            two_sum(fem, ez, fem_lo);
-            two_sum(fxy, xy, fxy_lo);
-        } else {
-            fem = __fadd2_rn(fem, ez);
-            fxy = __fadd2_rn(fxy, xy);
-        }
+        fem = __fadd2_rn(fem, make_float2(e, Sn.z));
+        fxy = __fadd2_rn(fxy, make_float2(Sn.x, Sn.y));
         if (a.alog && t < a.alog_mcs)
             a.alog[(int64_t)t * a.alog_stride + a.alog_base + (int64_t)r * a.n_sample_sites + q.orig] = ok ? 1 : 0;
     };
@@ -288,13 +269,7 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
             // long parts: shared memory goes to spins, so each warp adds its threads' sums, in FP64; the
             // first two steps halve the quantities per lane (six additions for the four)
             const int lane = tid & 31;
-            double v[4] = {(double)fem.x, (double)fxy.x, (double)fxy.y, (double)fem.y};
-            if (ta.long_runs) {
-                v[0] += (double)fem_lo.x;
-                v[1] += (double)fxy_lo.x;
-                v[2] += (double)fxy_lo.y;
-                v[3] += (double)fem_lo.y;
-            }
+            const double v[4] = {(double)fem.x, (double)fxy.x, (double)fxy.y, (double)fem.y};
             const bool hi = lane & 16, odd = lane & 8;
             double x = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xFFFFFFFFu, hi ? v[0] : v[2], 16);
             double y = (hi ? v[3] : v[1]) + __shfl_xor_sync(0xFFFFFFFFu, hi ? v[1] : v[3], 16);
@@ -305,7 +280,7 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
             if ((lane & 7) == 0) s_sum[(lane >> 3) * (NT >> 5) + (tid >> 5)] = x;
             if (lane == 0) s_num[tid >> 5] = n;
             bar_arrive(kBarFull, NT + kTileRecord);
-            fem = fxy = fem_lo = fxy_lo = make_float2(0.f, 0.f);
+            fem = fxy = make_float2(0.f, 0.f);
             nacc = 0;
             continue;
         }
@@ -315,24 +290,9 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
         o[NT] = fxy.x;
         o[2 * NT] = fxy.y;
         o[3 * NT] = fem.y;
-        if (ta.long_runs) {  // the errors are 2^-24 of the sums: one FP32 sum of them per warp
-            for (int off = 16; off > 0; off >>= 1) {
-                fem_lo = __fadd2_rn(fem_lo, make_float2(__shfl_xor_sync(0xFFFFFFFFu, fem_lo.x, off),
-                                                        __shfl_xor_sync(0xFFFFFFFFu, fem_lo.y, off)));
-                fxy_lo = __fadd2_rn(fxy_lo, make_float2(__shfl_xor_sync(0xFFFFFFFFu, fxy_lo.x, off),
-                                                        __shfl_xor_sync(0xFFFFFFFFu, fxy_lo.y, off)));
-            }
-            if ((tid & 31) == 0) {
-                float *l = s_lo + b * 4 * (NT >> 5) + (tid >> 5);
-                l[0] = fem_lo.x;
-                l[NT >> 5] = fxy_lo.x;
-                l[2 * (NT >> 5)] = fxy_lo.y;
-                l[3 * (NT >> 5)] = fem_lo.y;
-            }
-        }
         s_cnt[b * NT + tid] = nacc;
         bar_arrive(kBarFull + b, NT + kTileRecord);
-        fem = fxy = fem_lo = fxy_lo = make_float2(0.f, 0.f);
+        fem = fxy = make_float2(0.f, 0.f);
         nacc = 0;
     }
     bar_sync(kBarSweep, NT);
@@ -436,8 +396,8 @@ int32_t share(const TileShape &s, const TilePlan &out, int32_t c, int64_t p) {
 // Parts of compact regions: ranges of each class in memory order (a Morton curve when the sample
 // gives positions). When a part's share of a class is one round of threads, a part takes the
 // same places in every class and thread k of a block the k-th: it then adds the FP32 shares of
-// the sites that one thread of the other sweeps adds (site w of every class), in the same order, so
-// the histories agree to the FP64 sums' rounding.
+// site w of every class, in class order, as a thread of every sweep with a thread per site of the class
+// does, and the histories agree with that sweep's to the FP64 sums' rounding.
 bool tile_plan(const TileShape &s, TilePlan &out) {
     const int32_t n = s.n, nc = s.n_colours, P = s.parts;
     if (P < 1 || nc < 1) return false;
@@ -624,7 +584,7 @@ size_t tile_layout(TileArgs &a, const TilePlan &p, int threads) {
     at = align(at + (size_t)a.n_colours * sizeof(TileClass));
     a.part_off = (int32_t)at;
     if (a.mem == 0) return at + (size_t)(threads / 32) * (4 * sizeof(double) + sizeof(uint32_t));
-    return at + (size_t)(1 + a.two_buffers) * (threads * 5 + threads / 32 * 4) * sizeof(float);
+    return at + (size_t)(1 + a.two_buffers) * threads * 5 * sizeof(float);
 }
 
 }  // namespace
@@ -665,9 +625,6 @@ int tile_shape(TileArgs &a, const TileShape &s, TilePlan &p, size_t *smem) {
             return 0;
         // the last form gives up threads for spins (at least half of them)
         for (int nt = best; nt >= (a.mem == 0 ? std::min(best, kTileThreads / 2) : best) && !found; nt -= 32) {
-            // several attempts of a class per thread: in FP32 their sums' relative error falls as
-            // 1 / sqrt(n), and on small samples it is kept
-            a.long_runs = own > nt && s.n < 65536 ? 1 : 0;
             *smem = tile_layout(a, p, nt);
             int nb = 0;
             if (*smem + fa.sharedSizeBytes > (size_t)most) continue;
@@ -676,13 +633,15 @@ int tile_shape(TileArgs &a, const TileShape &s, TilePlan &p, size_t *smem) {
         }
     }
     if (!found) return 0;
+    p.columns = p.columns && own <= found;
     for (int32_t q = 0; q < s.parts; ++q) {  // a thread's FP32 sums: at most kTileRun attempts
-        int run = 0;
+        int32_t run = 0;
         for (int c = 0; c < a.n_colours; ++c) {
             const TileClass &cl = p.classes[(size_t)q * a.n_colours + c];
             run += (cl.end - cl.begin + found - 1) / found;
         }
         if (run > kTileRun) return 0;
+        p.run = std::max(p.run, run);
     }
     write_tables(a, s, p);
     return found;

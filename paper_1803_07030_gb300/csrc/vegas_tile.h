@@ -51,7 +51,6 @@ struct TileArgs {
     int32_t P, n_colours, n_mail, mcs, width;
     int32_t cubic;               // some site has a cubic constant
     int32_t skip_block;          // fault injection: this block never runs (-1: none)
-    int32_t long_runs;           // threads take several attempts of a class: compensated sums
     int32_t mem, n_codes, two_buffers;  // what is kept in shared memory (tile_shape)
     int32_t cap, rows_off, orig_off, pub_off, slot_off, code_off, cls_off, part_off;  // and where
 };
@@ -73,7 +72,8 @@ struct TilePlan {
     size_t row_bytes = 0;
     std::vector<float> codes;               // exchange values
     int32_t n_mail = 0, max_own = 0, max_halo = 0, max_loc = 0, widest = 0;
-    bool columns = false;
+    int32_t run = 0;                        // most attempts of one thread per MCS (tile_shape)
+    bool columns = false;                   // a thread takes one site of each class, the same place in all
 };
 
 // Adds the exchange values J[0..n), as far as kTileCodes goes, and padding's 0.
