@@ -1811,6 +1811,12 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
         NvtxRange run_range("vegas_run");
         c->probing = false;  // a timing that an error ended
         const int64_t nrec = (int64_t)n_steps * mcs;
+        const size_t hneed = (size_t)nrec * NI * 4, aneed = (size_t)nrec * NI;
+        RecordBlock rb;  // joins c->blocks when everything else has succeeded
+        rb.n = nrec;
+        rb.hist.reset(new double[hneed]);
+        rb.acc.reset(new uint32_t[aneed]);
+        if (c->blocks.size() == c->blocks.capacity()) c->blocks.reserve(2 * c->blocks.size() + 1);
         if (sched.size() > c->sched_cap) {
             if (c->d_sched) {
                 cudaFree(c->d_sched);
@@ -1820,7 +1826,6 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             CK(c, dalloc(c, &c->d_sched, sizeof(double) * sched.size()));
             c->sched_cap = sched.size();
         }
-        const size_t hneed = (size_t)nrec * NI * 4;
         if (hneed > c->hist_cap) {
             if (c->d_hist) {
                 cudaFree(c->d_hist);
@@ -1841,7 +1846,6 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             CK(c, dalloc(c, &c->d_acc_t, sizeof(uint32_t) * (hneed / 4)));
             c->hist_t_cap = hneed;
         }
-        const size_t aneed = (size_t)nrec * NI;
         if (aneed > c->acc_hist_cap) {
             if (c->d_acc_hist) {
                 cudaFree(c->d_acc_hist);
@@ -2174,10 +2178,6 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
         // records: [rec][inst] on the device, turned to [inst][rec] there, kept as one block per run
         // (256 nanoparticles x 1000 MCS: 0.3 ms after the sweep; copied record by record into
         // vectors per instance on the host, 9 ms)
-        RecordBlock rb;
-        rb.n = nrec;
-        rb.hist.reset(new double[hneed]);
-        rb.acc.reset(new uint32_t[aneed]);
         const double *src_h = c->d_hist;
         const uint32_t *src_a = c->d_acc_hist;
         if (NI > 1) {
@@ -2189,14 +2189,13 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
         CK(c, cudaMemcpyAsync(rb.hist.get(), src_h, sizeof(double) * hneed, cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaMemcpyAsync(rb.acc.get(), src_a, sizeof(uint32_t) * aneed, cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
-        c->blocks.push_back(std::move(rb));
-        if (tneed > 0) {  // [rec][inst][type][3] -> per instance, appended
+        if (tneed > 0) {  // [rec][inst][type][3] -> per instance, after the records there are
             std::vector<double> ht(tneed);
             CK(c, cudaMemcpy(ht.data(), c->d_type_hist, sizeof(double) * tneed, cudaMemcpyDeviceToHost));
             const size_t per = (size_t)c->n_types * 3;
             for (int64_t i = 0; i < NI; ++i) {
                 auto &v = c->type_hist[(size_t)i];
-                const size_t old = v.size();
+                const size_t old = (size_t)c->records * per;
                 v.resize(old + (size_t)nrec * per);
                 for (int64_t r = 0; r < nrec; ++r)
                     std::memcpy(&v[old + (size_t)r * per], &ht[((size_t)r * NI + i) * per], per * sizeof(double));
@@ -2210,7 +2209,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                 const SampleInfo &si = c->samples[(size_t)sm];
                 for (int32_t r = 0; r < c->R; ++r) {
                     auto &v = c->snaps[(size_t)(sm * c->R + r)];
-                    const size_t old = v.size();
+                    const size_t old = (size_t)c->snapshot_steps * (size_t)si.n * 3;
                     v.resize(old + (size_t)n_steps * (size_t)si.n * 3);
                     for (int32_t st = 0; st < n_steps; ++st)
                         for (int32_t g = 0; g < si.n; ++g) {
@@ -2233,9 +2232,11 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                         }
                 }
             }
-            c->snapshot_steps += n_steps;
         }
+        // nothing below throws: the records and their count change together
+        c->blocks.push_back(std::move(rb));
         c->records += nrec;
+        if (sneed > 0) c->snapshot_steps += n_steps;
         c->t += (uint32_t)nrec;
         c->device_error |= derr;
         if (derr & kErrTimeout)
@@ -2265,11 +2266,13 @@ template <typename F>
 void copy_records(const vegas_ctx *c, size_t bytes, void *out, F &&data) {
     auto some = [&](int i0, int i1) {
         for (int i = i0; i < i1; ++i) {
-            char *to = (char *)out + (size_t)i * (size_t)c->records * bytes;
+            size_t left = (size_t)c->records * bytes;  // of the instance's rows in out
+            char *to = (char *)out + (size_t)i * left;
             for (const RecordBlock &b : c->blocks) {
-                const size_t len = (size_t)b.n * bytes;
-                std::memcpy(to, (const char *)data(b) + (size_t)i * len, len);
+                const size_t row = (size_t)b.n * bytes, len = std::min(row, left);
+                std::memcpy(to, (const char *)data(b) + (size_t)i * row, len);
                 to += len;
+                left -= len;
             }
         }
     };
