@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kAnaThreads) thermal_tau_kernel(const ThermalA
     __shared__ int s_done;
     const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank(), lane = threadIdx.x & 31;
     const int64_t idx = blockIdx.x / CS, which = idx & 1, sid = idx >> 1, n = a.n;
-    const double *x = a.x + (which * a.n_series + sid) * a.stride;
+    double *x = a.x + (which * a.n_series + sid) * a.stride;
     const int64_t per = (n + CS - 1) / CS, i0 = rank * per, i1 = min(n, i0 + per);
     double v[kLags];
     auto total = [&](int buf) {  // lane q of a warp: the cluster's sum q, in rank order
@@ -259,9 +259,19 @@ __global__ void __launch_bounds__(kAnaThreads) thermal_tau_kernel(const ThermalA
             for (int b = 0; b < CS; ++b) t += cl.map_shared_rank(&s_blk[buf][0], b)[lane];
         return t;
     };
+    // The values were centred on the rounded plain mean: their own mean, added from the bins, goes too
+    // (a constant series is 0 only then). Each block takes it off its own records; the barrier shows the
+    // cluster's values to every block of it.
+    double rest = 0.0;
+    for (int b = lane; b <= a.n_bins; b += 32) rest += a.bins[(sid * (a.n_bins + 1) + b) * 8 + 2 * which];
+    rest = warp_sum(rest) / (double)n;
 #pragma unroll
     for (int q = 0; q < kLags; ++q) v[q] = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += kAnaThreads) v[0] += x[i] * x[i];
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += kAnaThreads) {
+        const double xi = x[i] - rest;
+        x[i] = xi;
+        v[0] += xi * xi;
+    }
     block_sums<kLags>(v, sm, s_blk[0]);
     if (threadIdx.x == 0) {
         s_tau = 0.5;

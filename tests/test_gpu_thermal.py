@@ -49,3 +49,14 @@ def test_constant_series_has_no_correlation_time():
     H = np.tile(np.array([-5.0, 0.0, 3.0, 4.0]), (2, 100, 1))
     out = vg.thermal_averages(H, 10, 5, 1.0, 10.0)
     assert np.allclose(out[:, [12, 13]], 0.5) and np.allclose(out[:, 0], -0.5) and np.allclose(out[:, 2], 0.5)
+
+
+def test_constant_series_whose_sum_rounds():
+    """n equal values whose sum is rounded have another plain mean: what is left after centring is zero."""
+    rng = np.random.default_rng(7)
+    for n, bins, values in ((8000, 20, (-1689.6, -921.6)), (800, 20, (-921.6, -0.1)), (1237, 10, tuple(-rng.uniform(1, 9e4, 60)))):
+        H = np.empty((len(values), n, 4))
+        H[:, :, 0] = np.array(values)[:, None]
+        H[:, :, 1:] = (np.array(values) * 0.7)[:, None, None] * np.array([0.36, 0.48, 0.8])
+        out = vg.thermal_averages(H, 0, bins, 1.3, 4096.0)
+        assert np.array_equal(out[:, [12, 13]], np.full((len(values), 2), 0.5))
