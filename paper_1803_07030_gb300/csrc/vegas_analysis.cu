@@ -118,7 +118,8 @@ __device__ __forceinline__ void series_means(const ThermalArgs &a, int64_t sid, 
 }
 
 // Centred values e' = E - Eref, a' = |M| - Aref of one bin (block n_bins: the records behind the
-// bins), in place, and their moments: sums of e', e'^2, a', a'^2, a' e', M^2, M^4, M^2 e'.
+// bins), in place, and their moments: sums of e', e'^2, a', a'^2, a' e', M^2, M^4, M^2 e'. M^2 comes
+// from the components, not from the rounded |M|.
 __global__ void __launch_bounds__(kAnaThreads) thermal_bin_kernel(const ThermalArgs a) {
     __shared__ double sm[8][kAnaThreads], s_out[8], s_ref[2];
     const int64_t sid = blockIdx.y, b = a.n / a.n_bins;
@@ -133,11 +134,13 @@ __global__ void __launch_bounds__(kAnaThreads) thermal_bin_kernel(const ThermalA
     __syncthreads();
     const double Eref = s_ref[0], Aref = s_ref[1];
     double *xe = a.x + sid * a.stride, *xa = a.x + (a.n_series + sid) * a.stride;
+    const double2 *h = (const double2 *)(a.series + (sid * a.len + a.cut) * 4);
     const bool rest = (int)blockIdx.x == a.n_bins;
     const int64_t i0 = blockIdx.x * b, i1 = rest ? a.n : i0 + b;
     double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int64_t i = i0 + threadIdx.x; i < i1; i += kAnaThreads) {
-        const double m = xa[i], m2 = m * m, e = xe[i] - Eref, d = m - Aref;
+        const double2 p = h[2 * i], q = h[2 * i + 1];
+        const double m2 = p.y * p.y + q.x * q.x + q.y * q.y, e = xe[i] - Eref, d = xa[i] - Aref;
         xe[i] = e;
         xa[i] = d;
         v[0] += e;

@@ -60,3 +60,13 @@ def test_constant_series_whose_sum_rounds():
         H[:, :, 1:] = (np.array(values) * 0.7)[:, None, None] * np.array([0.36, 0.48, 0.8])
         out = vg.thermal_averages(H, 0, bins, 1.3, 4096.0)
         assert np.array_equal(out[:, [12, 13]], np.full((len(values), 2), 0.5))
+
+
+def test_squares_come_from_the_components():
+    """M^2 of 2 and 12, whose roots round: 72 and 4 of 128 records (the others 0) give U4 = 0 exactly."""
+    H = np.zeros((1, 128, 4))
+    H[0, :, 0] = np.arange(128) % 3
+    H[0, :72, 1:3] = 1.0
+    H[0, 72:76, 1:] = 2.0
+    out = vg.thermal_averages(H, 0, 4, 1.0, 10.0)
+    assert out[0, vg.AVG_FIELDS.index("u4")] == 0.0
