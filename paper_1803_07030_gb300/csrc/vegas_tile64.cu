@@ -30,9 +30,17 @@ namespace {
 
 constexpr int kBarSweep = 1, kBarFull = 2, kBarEmpty = 4;  // as in vegas_tile.cu
 constexpr unsigned kAll = 0xFFFFFFFFu;
-constexpr uint32_t kTile64Spins = 1u << 26;  // polls of a wait inside the block (seconds) before it gives up
 
 __device__ __forceinline__ float as_f(uint32_t x) { return __uint_as_float(x); }
+
+// Whether a wait of one part of the block for another has run out at its n-th poll: that part may
+// itself wait timeout_ns for a remote word, so after twice that and a second.
+__device__ __forceinline__ bool inner_wait_over(uint32_t n, uint64_t &since, int64_t timeout_ns) {
+    if ((n & 1023u) != 0) return false;
+    const uint64_t now = tile_ns();
+    if (since == 0) since = now;
+    return (now - since) / 2 > (uint64_t)timeout_ns + 500000000u;
+}
 
 // W: links per fixed row (6 or kEllRow; padded with links of J = 0 to the site itself). PM: 0 no
 // anisotropy and uniform parameters, else 2.
@@ -123,14 +131,21 @@ __global__ void __launch_bounds__(kTile64Threads + kTile64Trial + 32) tile64_ker
         const int w = (tid - NT) >> 5;
         const int64_t total = (int64_t)tt.mcs * nc;
         for (int64_t seq = w; seq < total; seq += kTile64Trial / 32) {
-            for (uint32_t n = 0; (int)seq - s_used >= kTile64Ahead; ++n) {
-                if (s_ok == 0) return;
-                if (n > kTile64Spins) {  // the sweeping warps wait in turn, with the same limit
-                    if (lane == 0) atomicOr(a.err, kErrTimeout);
-                    return;
+            int go = 1;
+            uint64_t since = 0;
+            if (lane == 0)  // one lane waits for all: they leave together
+                for (uint32_t n = 1; go && (int)seq - s_used >= kTile64Ahead; ++n) {
+                    if (s_ok == 0) {
+                        go = 0;
+                    } else if (inner_wait_over(n, since, tt.timeout_ns)) {  // the sweeping warps give up in turn
+                        atomicOr(a.err, kErrTimeout);
+                        go = 0;
+                    } else {
+                        __nanosleep(40);
+                    }
                 }
-                __nanosleep(40);
-            }
+            __syncwarp();
+            if (!__shfl_sync(kAll, go, 0)) return;
             const int c = (int)(seq % nc), slot = (int)(seq % kTile64Ahead);
             const uint32_t t = t0 + (uint32_t)(seq / nc);
             const TileClass cl = s_cls[c];
@@ -294,12 +309,11 @@ __global__ void __launch_bounds__(kTile64Threads + kTile64Trial + 32) tile64_ker
             const TileClass cl = s_cls[c];
             const int slot = seq % kTile64Ahead;
             bool drawn = true;  // the trial warps run classes ahead
-            for (uint32_t n = 0; s_ready[slot] != seq + 1; ++n)
-                if (n > kTile64Spins) {
-                    atomicOr(a.err, kErrTimeout);
-                    drawn = false;
-                    break;
-                }
+            if (s_ready[slot] != seq + 1) {
+                uint64_t since = 0;
+                for (uint32_t n = 1; drawn && s_ready[slot] != seq + 1; ++n) drawn = !inner_wait_over(n, since, tt.timeout_ns);
+                if (!drawn) atomicOr(a.err, kErrTimeout);
+            }
             __threadfence_block();
             const int n_cls = cl.end - cl.begin;
             int j = my;
