@@ -1182,7 +1182,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
                 const int64_t per_sm = (work + c->sm_count - 1) / c->sm_count;
                 pl.threads = (int)std::min<int64_t>(kThreads, std::max<int64_t>(32, (per_sm + 31) / 32 * 32));
             }
-            if (c->precision != 64) pl.threads = pass32_threads(a);  // the R = 32 kernel runs 7-warp blocks
+            if (c->precision != 64) pl.threads = pass32_threads(a);  // the R = 32 kernel's own blocks
             const int64_t need = (work + pl.threads - 1) / pl.threads;
             int64_t cap = (int64_t)c->sm_count * pass_blocks_per_sm(c->precision, a);
             if (o.max_blocks > 0) cap = std::min<int64_t>(cap, o.max_blocks);
@@ -1890,6 +1890,7 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
         rs.type_hist = c->n_types > 0 ? c->d_type_hist : nullptr;
         rs.rec_end = (uint32_t)nrec;
         CK(c, cudaMemcpyAsync(c->d_run, &rs, sizeof rs, cudaMemcpyHostToDevice, c->stream));
+        if (c->tile_ok) CK(c, cudaMemsetAsync(c->tile.abort, 0, sizeof(uint32_t), c->stream));
 
         const bool use_graph = c->opt.graphs != 0 && !c->opt.timing;
         if (use_graph && (st = build_graph(c)) != VEGAS_OK) return st;
@@ -2243,7 +2244,9 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             return fail(c, VEGAS_ETIMEOUT,
                         c->variant == 4 ? "a warp of the wavefront sweep waited longer than timeout_ns for the class-0 "
                                           "blocks that a class-1 block links to"
-                                        : "a grid barrier of the cooperative sweep waited longer than timeout_ns");
+                        : c->use_tile ? "a block of the tiled cooperative sweep waited longer than timeout_ns for a boundary "
+                                        "spin of another block"
+                                      : "a grid barrier of the cooperative sweep waited longer than timeout_ns");
         if (derr) {
             char msg[200];
             std::snprintf(msg, sizeof msg,

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
     __shared__ int s_ok;  // 0: the record warp leaves
     RunState *rs = a.run;
     const uint32_t t0 = rs->t, rec0 = rs->rec;
-    if (tid == 0) s_ok = 1;
+    if (tid == 0) s_ok = *(volatile uint32_t *)ta.abort == 0u ? 1 : 0;
     for (int c = tid; c < nc; c += blockDim.x) s_cls[c] = ta.classes[part * nc + c];
     const float4 *S = (const float4 *)a.spins;
     for (int k = tid; k < pt.n_own + pt.n_halo; k += blockDim.x) {
@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(cons
     if (FMT == 1)
         for (int k = tid; k < ta.n_codes; k += blockDim.x) s_J[k] = ta.codes[k];
     __syncthreads();
+    if (s_ok == 0) return;  // a wait of an earlier launch of the run ran out
     if (tid >= NT) {
         // record warp q: the total of quantity q over the sweeping threads after every MCS, in a
         // fixed order in FP64 (and, in warp 0, the accepted attempts)
@@ -652,7 +653,6 @@ int launch_tile(const TileArgs &a, int threads, size_t smem, void *stream) {
     // no word may carry a tag of this launch before it is stored (the MCS counter can be set back)
     cudaError_t e = cudaMemsetAsync(a.mail, 0, ((size_t)a.n_mail << a.pass.log2R) * sizeof(float4), st);
     if (e != cudaSuccess) return (int)e;
-    if ((e = cudaMemsetAsync(a.abort, 0, sizeof(uint32_t), st)) != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.P << a.pass.log2R));
     cfg.blockDim = dim3((unsigned)(threads + kTileRecord));

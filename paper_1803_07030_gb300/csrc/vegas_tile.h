@@ -45,7 +45,7 @@ struct TileArgs {
     float4 *mail;                // [R][n_mail] (x, y, z, MCS counter + 1)
     double *partial;             // [mcs][R][4][P]
     uint32_t *count;             // [mcs][R][P] accepted attempts
-    uint32_t *abort;             // set when a wait ran out: every block leaves
+    uint32_t *abort;             // set when a wait ran out: every block leaves, as do the run's later launches
     int64_t timeout_ns;
     uint32_t rk0[10], rk1[10];   // Philox round keys
     int32_t P, n_colours, n_mail, mcs, width;

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kTile64Threads + kTile64Trial + 32) tile64_ker
     RunState *rs = a.run;
     const uint32_t t0 = rs->t, rec0 = rs->rec;
     if (tid == 0) {
-        s_ok = 1;
+        s_ok = *(volatile uint32_t *)tt.abort == 0u ? 1 : 0;
         s_used = 0;
     }
     if (tid < kTile64Ahead) s_ready[tid] = 0;
@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(kTile64Threads + kTile64Trial + 32) tile64_ker
         s_J[k] = __ldg(ta.J + (int64_t)pt.own_begin * W + k);
     }
     __syncthreads();
+    if (s_ok == 0) return;  // a wait of an earlier launch of the run ran out
     const uint32_t inst = (uint32_t)(a.inst0 + r);
     const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
     if (tid >= NT + kTile64Trial) {
@@ -431,7 +432,6 @@ int launch_tile64(const Tile64Args &a, int threads, size_t smem, void *stream) {
     // no word may carry a tag of this launch before it is stored (the MCS counter can be set back)
     cudaError_t e = cudaMemsetAsync(t.mail, 0, ((size_t)t.n_mail << t.pass.log2R) * 2 * sizeof(float4), st);
     if (e != cudaSuccess) return (int)e;
-    if ((e = cudaMemsetAsync(t.abort, 0, sizeof(uint32_t), st)) != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(t.P << t.pass.log2R));
     cfg.blockDim = dim3((unsigned)(threads + kTile64Trial + 32));
