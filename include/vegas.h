@@ -230,7 +230,10 @@ typedef struct {
     double last_run_ms;         /* event time of the last vegas_run on the device */
     int64_t device_bytes;       /* device memory held by the context */
     int32_t n_types;            /* site types tracked per instance (type_stats), else 0 */
-    int32_t pad_;
+    int32_t tile_form;          /* cooperative sweep in use: 0 its grid-barrier form; otherwise the
+                                   tiled one: 1, + 2 x what a block keeps in shared memory beside the
+                                   spins (2 rows and site ids, 1 ids, 0 nothing), + 8 rows of words,
+                                   + 16 a thread takes one site of each class (FP64: 1) */
     int64_t snapshot_steps;     /* steps with a stored final state per instance (snapshots) */
     int32_t block_threads;      /* threads per block of the sweep in use (the resident sweep's
                                    is chosen by the autotuner: 256 or 512) */

@@ -2521,6 +2521,9 @@ extern "C" vegas_status vegas_stats(const vegas_ctx *c, vegas_stats_t *o) {
         o->block_threads = c->variant == 1 ? c->res_threads : (c->variant == 3 ? c->cluster_threads : kThreads);
         if (c->variant == 2 && c->use_tile)
             o->block_threads = c->tile_threads + (c->precision == 64 ? kTile64Trial + 32 : kTileRecord);
+        if (c->variant == 2 && c->use_tile)
+            o->tile_form = c->precision == 64 ? 1
+                                              : 1 + 2 * c->tile.mem + (c->tile.n_codes ? 8 : 0) + (c->tile_order.columns ? 16 : 0);
         o->cluster_blocks = c->variant == 3 ? c->cluster_cs : 0;
         o->split_sites = c->variant == 3 ? c->res.split_sites : 0;
         o->group_threads = (c->variant == 1 || c->variant == 3) ? c->res.group_threads : 0;

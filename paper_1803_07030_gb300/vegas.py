@@ -108,7 +108,7 @@ class vegas_stats_t(C.Structure):
         ("last_run_ms", C.c_double),
         ("device_bytes", C.c_int64),
         ("n_types", C.c_int32),
-        ("pad_", C.c_int32),
+        ("tile_form", C.c_int32),
         ("snapshot_steps", C.c_int64),
         ("block_threads", C.c_int32),
         ("cluster_blocks", C.c_int32),
