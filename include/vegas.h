@@ -165,7 +165,9 @@ typedef struct {
     int32_t fault_inject;   /* testing only: 1 = in the cooperative sweep one block leaves
                                before its first grid barrier, and in the wavefront sweep the
                                first block of class-0 sites is never reported finished, so the
-                               blocks that wait for it time out. Default 0. */
+                               blocks that wait for it time out; 2 = device buffers that only make
+                               runs faster are not allocated, as when device memory is short.
+                               Default 0. */
     int32_t type_stats;     /* 1: also record the magnetization of every site type (magnetic
                                phase, Sec. II) after every MCS (vegas_type_history). Sites are
                                then stored type by type inside each colour class, and the

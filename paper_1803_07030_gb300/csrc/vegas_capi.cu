@@ -87,7 +87,7 @@ struct vegas_ctx {
     // device buffers
     void *d_spins = nullptr, *d_edges = nullptr, *d_p0 = nullptr, *d_p1 = nullptr, *d_pk = nullptr;
     int2 *d_ell = nullptr;  // links as fixed rows of kEllRow (spins-in-shared-memory sweeps)
-    void *d_batch_rows = nullptr;  // rows, exchange values and lower modes of batch32_kernel
+    void *d_batch_rows = nullptr;  // rows, exchange values and lower modes of batch32_kernel, one allocation
     float *d_batch_codes = nullptr;
     int32_t *d_batch_modes = nullptr;
     int64_t *d_rowptr = nullptr, *d_slot_base = nullptr;
@@ -102,8 +102,7 @@ struct vegas_ctx {
     int32_t *d_orig = nullptr, *d_slot_count = nullptr;
     double *d_norm = nullptr, *d_partial = nullptr, *d_sched = nullptr, *d_hist = nullptr;
     size_t sched_cap = 0, hist_cap = 0;
-    double *d_hist_t = nullptr;  // the run's records by instance
-    uint32_t *d_acc_t = nullptr;
+    double *d_hist_t = nullptr;  // the run's records by instance, then their accepted attempts
     size_t hist_t_cap = 0;
     // acceptance counts and update policies
     uint32_t *d_acc = nullptr, *d_acc_hist = nullptr;
@@ -237,14 +236,24 @@ cudaError_t dalloc(vegas_ctx *c, T **p, size_t bytes) {
     return e;
 }
 
+// A buffer that only makes runs faster: *p is NULL when there is no memory for it.
+template <typename T>
+cudaError_t dalloc_spare(vegas_ctx *c, T **p, size_t bytes) {
+    *p = nullptr;
+    const cudaError_t e = c->opt.fault_inject == 2 ? cudaErrorMemoryAllocation : dalloc(c, p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return cudaSuccess;
+}
+
 void free_all(vegas_ctx *c) {
     for (auto &kv : c->step_graphs) cudaGraphExecDestroy(kv.second);
     for (auto &kv : c->run_graphs) cudaGraphExecDestroy(kv.second);
     for (cudaGraph_t g : c->run_graph_defs) cudaGraphDestroy(g);
     if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
     if (c->graph) cudaGraphDestroy(c->graph);
-    void *bufs[] = {c->d_spins, c->d_edges, c->d_ell, c->d_batch_rows, c->d_batch_codes, c->d_batch_modes, c->d_p0, c->d_p1, c->d_pk, c->d_rowptr, c->d_slot_base, c->d_orig,
-                    c->d_slot_count, c->d_norm, c->d_partial, c->d_sched, c->d_hist, c->d_hist_t, c->d_acc_t, c->d_run, c->d_err, c->d_alog,
+    void *bufs[] = {c->d_spins, c->d_edges, c->d_ell, c->d_batch_rows, c->d_p0, c->d_p1, c->d_pk, c->d_rowptr, c->d_slot_base, c->d_orig,
+                    c->d_slot_count, c->d_norm, c->d_partial, c->d_sched, c->d_hist, c->d_hist_t, c->d_run, c->d_err, c->d_alog,
                     c->d_insts, c->d_cstart, c->d_queue, c->d_bar, c->d_coop_partial, c->d_acc, c->d_acc_hist,
                     c->d_pol, c->d_pol32, c->d_qis, c->d_sigma, c->d_adapt_n, c->d_type_hist, c->d_snap, c->d_segs,
                     c->d_tasks, c->d_deps, c->d_done, c->d_ticket, c->d_pass_tickets, c->d_wave_partial, c->d_wave_slot_base, c->d_wave_slot_count,
@@ -744,7 +753,8 @@ vegas_status make_tile(vegas_ctx *c, const LoadedSample &l) {
     size_t total = 0;
     for (const Table &t : tables) total += (std::max<size_t>(t.bytes, 16) + 255) / 256 * 256;
     unsigned char *mem = nullptr;
-    CK(c, dalloc(c, &mem, total));
+    CK(c, dalloc_spare(c, &mem, total));
+    if (!mem) return VEGAS_OK;  // the other sweeps need no such tables
     c->tile_bufs.push_back(mem);
     for (const Table &t : tables) {
         *t.at = mem;
@@ -823,7 +833,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         return fail(nullptr, VEGAS_EINVAL, "cluster_threads must be 0, 256 or 512");
     if (o.variant == 3 && o.precision != 32)
         return fail(nullptr, VEGAS_EINVAL, "the cluster sweep (variant 3) is FP32 only");
-    if (o.timeout_ns < 0 || o.fault_inject < 0 || o.fault_inject > 1) return fail(nullptr, VEGAS_EINVAL, "bad timeout or fault_inject");
+    if (o.timeout_ns < 0 || o.fault_inject < 0 || o.fault_inject > 2) return fail(nullptr, VEGAS_EINVAL, "bad timeout or fault_inject");
     if (o.graphs < 0 || o.graphs > 2) return fail(nullptr, VEGAS_EINVAL, "graphs must be 0, 1 or 2");
     if (o.type_stats < 0 || o.type_stats > 1 || o.snapshots < 0 || o.snapshots > 1)
         return fail(nullptr, VEGAS_EINVAL, "type_stats and snapshots must be 0 or 1");
@@ -1389,12 +1399,22 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
                 ba.rk0[q] = (uint32_t)o.seed + q * 0x9E3779B9u;
                 ba.rk1[q] = (uint32_t)(o.seed >> 32) + q * 0xBB67AE85u;
             }
-            DALLOC(c->d_batch_rows, sizeof(uint32_t) * h_rows.size());
-            DALLOC(c->d_batch_codes, sizeof(float) * h_codes.size());
-            DALLOC(c->d_batch_modes, sizeof(int32_t) * std::max<size_t>(h_modes.size(), 1));
-            H2D(c->d_batch_rows, h_rows.data(), sizeof(uint32_t) * h_rows.size());
-            H2D(c->d_batch_codes, h_codes.data(), sizeof(float) * h_codes.size());
-            if (!h_modes.empty()) H2D(c->d_batch_modes, h_modes.data(), sizeof(int32_t) * h_modes.size());
+            unsigned char *mem = nullptr;  // one allocation for the three tables
+            const size_t row_b = (sizeof(uint32_t) * h_rows.size() + 255) / 256 * 256;
+            const size_t code_b = (sizeof(float) * h_codes.size() + 255) / 256 * 256;
+            if (dalloc_spare(c, &mem, row_b + code_b + sizeof(int32_t) * std::max<size_t>(h_modes.size(), 1)) != cudaSuccess) {
+                c->err = "cudaMalloc of the sweep tables failed";
+                return bail(VEGAS_ECUDA);
+            }
+            c->batch_ok = mem != nullptr;  // the former kernels do without
+            c->d_batch_rows = mem;
+            if (mem) {
+                c->d_batch_codes = (float *)(mem + row_b);
+                c->d_batch_modes = (int32_t *)(mem + row_b + code_b);
+                H2D(c->d_batch_rows, h_rows.data(), sizeof(uint32_t) * h_rows.size());
+                H2D(c->d_batch_codes, h_codes.data(), sizeof(float) * h_codes.size());
+                if (!h_modes.empty()) H2D(c->d_batch_modes, h_modes.data(), sizeof(int32_t) * h_modes.size());
+            }
             ba.rows = c->d_batch_rows;
             ba.codes = c->d_batch_codes;
             ba.modes = c->d_batch_modes;
@@ -1835,17 +1855,6 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             CK(c, dalloc(c, &c->d_hist, sizeof(double) * hneed));
             c->hist_cap = hneed;
         }
-        if (NI > 1 && hneed > c->hist_t_cap) {  // the same records by instance
-            for (void *p : {(void *)c->d_hist_t, (void *)c->d_acc_t})
-                if (p) cudaFree(p);
-            c->d_hist_t = nullptr;
-            c->d_acc_t = nullptr;
-            c->device_bytes -= (int64_t)(c->hist_t_cap * sizeof(double) + c->hist_t_cap / 4 * sizeof(uint32_t));
-            c->hist_t_cap = 0;
-            CK(c, dalloc(c, &c->d_hist_t, sizeof(double) * hneed));
-            CK(c, dalloc(c, &c->d_acc_t, sizeof(uint32_t) * (hneed / 4)));
-            c->hist_t_cap = hneed;
-        }
         if (aneed > c->acc_hist_cap) {
             if (c->d_acc_hist) {
                 cudaFree(c->d_acc_hist);
@@ -1875,6 +1884,15 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             c->snap_cap = 0;
             CK(c, dalloc(c, &c->d_snap, sneed));
             c->snap_cap = sneed;
+        }
+        if (NI > 1 && hneed > c->hist_t_cap) {  // the same records by instance, where there is room for them
+            if (c->d_hist_t) {
+                cudaFree(c->d_hist_t);
+                c->device_bytes -= (int64_t)(c->hist_t_cap * sizeof(double) + c->hist_t_cap / 4 * sizeof(uint32_t));
+            }
+            c->hist_t_cap = 0;
+            CK(c, dalloc_spare(c, &c->d_hist_t, sizeof(double) * hneed + sizeof(uint32_t) * aneed));
+            if (c->d_hist_t) c->hist_t_cap = hneed;
         }
         CK(c, cudaMemcpyAsync(c->d_sched, sched.data(), sizeof(double) * sched.size(), cudaMemcpyHostToDevice, c->stream));
         RunState rs{};
@@ -2181,15 +2199,27 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
         // vectors per instance on the host, 9 ms)
         const double *src_h = c->d_hist;
         const uint32_t *src_a = c->d_acc_hist;
-        if (NI > 1) {
-            launch_by_instance(c->d_hist, c->d_acc_hist, c->d_hist_t, c->d_acc_t, NI, nrec, c->stream);
+        if (NI > 1 && c->d_hist_t) {
+            uint32_t *acc_t = (uint32_t *)(c->d_hist_t + hneed);
+            launch_by_instance(c->d_hist, c->d_acc_hist, c->d_hist_t, acc_t, NI, nrec, c->stream);
             CK(c, cudaGetLastError());
             src_h = c->d_hist_t;
-            src_a = c->d_acc_t;
+            src_a = acc_t;
         }
         CK(c, cudaMemcpyAsync(rb.hist.get(), src_h, sizeof(double) * hneed, cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaMemcpyAsync(rb.acc.get(), src_a, sizeof(uint32_t) * aneed, cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
+        if (NI > 1 && !c->d_hist_t) {  // turned here
+            RecordBlock by_rec = std::move(rb);
+            rb.n = nrec;
+            rb.hist.reset(new double[hneed]);
+            rb.acc.reset(new uint32_t[aneed]);
+            for (int64_t r = 0; r < nrec; ++r)
+                for (int64_t i = 0; i < NI; ++i) {
+                    std::memcpy(&rb.hist[((size_t)i * nrec + r) * 4], &by_rec.hist[((size_t)r * NI + i) * 4], 4 * sizeof(double));
+                    rb.acc[(size_t)i * nrec + r] = by_rec.acc[(size_t)r * NI + i];
+                }
+        }
         if (tneed > 0) {  // [rec][inst][type][3] -> per instance, after the records there are
             std::vector<double> ht(tneed);
             CK(c, cudaMemcpy(ht.data(), c->d_type_hist, sizeof(double) * tneed, cudaMemcpyDeviceToHost));
