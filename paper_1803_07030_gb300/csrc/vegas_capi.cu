@@ -1349,7 +1349,9 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         for (int64_t g = 0; g < n_sites; ++g) max_deg = std::max(max_deg, h_rowptr[(size_t)g + 1] - h_rowptr[(size_t)g]);
         c->res_smem_eligible = o.resident_smem >= 0 && 12 * (int64_t)c->max_instance_sites <= kResSmemBytes &&
                                max_deg <= kEllRow;
-        c->batch_ok = c->res_smem_eligible && !any_policy && c->n_types == 0;
+        // the tables of the shared-memory forms, where the context may run them
+        const bool smem_forms = c->res_smem_eligible && (o.variant < 0 || o.resident_smem == 1);
+        c->batch_ok = smem_forms && !any_policy && c->n_types == 0;
         std::vector<int2> h_ell;           // outlive the uploads below
         std::vector<uint32_t> h_rows;
         std::vector<float> h_codes;
@@ -1421,7 +1423,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         }
         // the forms with policies or per-type sums, blocks of 256 or groups of 64 threads when asked for, and
         // the autotuner's timings
-        if (c->res_smem_eligible) {
+        if (smem_forms) {
             h_ell.assign((size_t)n_sites * kEllRow, make_int2(-1, 0));
             host_ranges(n_sites, (int32_t)std::min<int64_t>(16, n_sites / 32768 + 1), [&](int64_t g0, int64_t g1) {
                 for (int64_t g = g0; g < g1; ++g)
@@ -1497,7 +1499,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
         // (the resident sweep's, or built here), read without row offsets
         const int deg0 = c->passes[0].args.deg;
         bool use_ell = false;
-        TRY(make_tile(c, L[0]));
+        if (o.variant < 0 || o.variant == 2) TRY(make_tile(c, L[0]));
         if (!p64 && deg0 != 6) {
             int64_t max_deg = 0;
             for (int64_t g = 0; g < n_sites; ++g)
