@@ -1351,7 +1351,7 @@ static vegas_status create_context(const vegas_sample *samples, int32_t n_sample
                                max_deg <= kEllRow;
         // the tables of the shared-memory forms, where the context may run them
         const bool smem_forms = c->res_smem_eligible && (o.variant < 0 || o.resident_smem == 1);
-        c->batch_ok = smem_forms && !any_policy && c->n_types == 0;
+        c->batch_ok = smem_forms && !any_policy && c->n_types == 0 && c->max_colours <= kBatchColours;
         std::vector<int2> h_ell;           // outlive the uploads below
         std::vector<uint32_t> h_rows;
         std::vector<float> h_codes;

@@ -124,6 +124,9 @@ int launch_tile64(const Tile64Args &a, int threads, size_t smem, void *stream);
 
 // ---- batches with spins in shared memory (vegas_batch.cu)
 constexpr int kBatchThreads = 512;    // sweeping threads per block
+constexpr int kBatchColours = 30;     // most colour classes: a thread's FP32 sums of one MCS are then at most 64
+                                      // attempts (spins in shared memory leave at most 34 sites per thread,
+                                      // and one more per class), one run of the former kernels
 
 struct BatchArgs {
     ResidentArgs r;

@@ -76,3 +76,17 @@ def test_batches_of_different_sizes_in_turn():
             a.run(1.0, 0.0, 4)
             c.run(1.0, 0.0, 4)
         assert np.array_equal(b.spins(1), c.spins(1))
+
+
+def test_many_classes_keep_the_former_sums():
+    """62 colour classes, 91 attempts per thread and MCS: the former kernels end a run of FP32 sums at 64."""
+    s = sc_periodic((20, 20, 40))
+    parity = np.asarray(vg.vegas_greedy_colour(s.row_ptr, s.col)[0])
+    s.colour = np.where(np.arange(s.n_sites) < 60, 2 + np.arange(s.n_sites), parity).astype(np.int32)
+    got = []
+    for fault in (0, 2):  # 2: without the batch kernel's tables
+        with vg.Context([s], seed=3, variant=1, resident_smem=1, fault_inject=fault, stream=None) as c:
+            c.run(1.0, 0.1, 6)
+            got.append((c.history(), c.spins(0)))
+    assert np.array_equal(got[0][1], got[1][1])
+    assert np.abs(got[0][0] - got[1][0]).max() <= 2.0 ** -50 * 8.0 * s.n_sites  # FP64 sums in another order
