@@ -200,10 +200,17 @@ __global__ void __launch_bounds__(R32Shape<POL>::WARPS * 32, R32Shape<POL>::MIN_
             if (g < g_end) {
                 const unsigned char *slot = lslots + ls * SLOT;
                 const uint32_t orig = ((const uint32_t *)(slot + LINK_BYTES))[j];
-                staged_attempt<DEG, PM, LM, POL, RN != 0>(a, (const int4 *)slot + j * (DEG / 2),
-                                                 PlanarRows{(const float *)(wbase + (j & 1) * (DEG + 1) * Sh::ROW), lane}, orig, g, r, R, t, inst, a.rk0, a.rk1,
-                                                 beta, B, S, acc, nan_seen, log_accepts,
-                                                 (const PolicySite32 *)(slot + POL_OFF) + j, sigma);
+                uint4 rw = make_uint4(orig, t, inst, kPurposeTrial32);
+#pragma unroll
+                for (int q = 0; q < 10; ++q) {  // Philox with the round keys as kernel arguments, by constant index
+                    const uint32_t lo0 = 0xD2511F53u * rw.x, hi0 = __umulhi(0xD2511F53u, rw.x);
+                    const uint32_t lo1 = 0xCD9E8D57u * rw.z, hi1 = __umulhi(0xCD9E8D57u, rw.z);
+                    rw = make_uint4(hi1 ^ rw.y ^ a.rk0[q], lo1, hi0 ^ rw.w ^ a.rk1[q], lo0);
+                }
+                staged_attempt_rw<DEG, PM, LM, POL, RN != 0>(
+                    a, (const int4 *)slot + j * (DEG / 2),
+                    PlanarRows{(const float *)(wbase + (j & 1) * (DEG + 1) * Sh::ROW), lane}, orig, g, r, R, t, rw, beta, B, S,
+                    acc, nan_seen, log_accepts, (const PolicySite32 *)(slot + POL_OFF) + j, sigma);
             }
             __syncwarp();
             if (j == 0 && lane == 0) tk = atomicAdd(a.ticket, 1u);
