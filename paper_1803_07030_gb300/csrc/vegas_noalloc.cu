@@ -310,7 +310,10 @@ extern "C" vegas_status vegas_sweep_noalloc(void *spins, const void *links, cons
         ReduceArgs ra{partial, hdr->slot_base, hdr->slot_count, &hdr->run, nullptr, replicas, replicas, 1, 0, nullptr, 0};
         launch_reduce(ra, st);
         e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
+        if (e != cudaSuccess) {
+            cudaStreamSynchronize(st);  // launches before the one refused may still write err_word
+            return fail(VEGAS_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
+        }
         e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return fail(VEGAS_ECUDA, std::string("sweep: ") + cudaGetErrorString(e));
         if (a.err == &err_word) return sweep_status(*(volatile uint32_t *)&err_word);
