@@ -45,6 +45,8 @@ L_DEPTH = 0  # z extent of the lattice, 0: the side (profiling cases may be flat
 # algorithmic bytes per attempt: 16 B read + 16 B write of the FP32 spin (float4), plus one
 # row of six (int32 col, f32 J) links = 48 B shared by the 32 replicas that sweep it together
 BYTES_PER_ATTEMPT = 16 + 16 + 48.0 / REPLICAS
+# what the kernel of 32 replicas has to move: its rows keep three of the four floats
+ROW_BYTES_PER_ATTEMPT = 12 + 12 + 48.0 / REPLICAS
 CSRC = os.path.join(ROOT, "paper_1803_07030_gb300", "csrc")
 # per sweep variant: the kernel that sweeps, its committed ncu summary, the sources it is built
 # from (the summary's counters are used only while their hash matches), and how many colour
@@ -496,6 +498,7 @@ def run_ours(args):
     attempts_per_launch = REPLICAS * s.n_sites * kclasses // 2
     peak, peak_kind = peaks()
     achieved = BYTES_PER_ATTEMPT * attempts_per_launch / (sweep_ms / 1000.0) / 1e9
+    row_bytes = ROW_BYTES_PER_ATTEMPT if kname == "pass32_r32" else BYTES_PER_ATTEMPT
     # the committed counters are those of the 256^3 workload; another side has none
     traffic = profiled_traffic(ksummary, ksources) if L_SIDE == 256 and L_DEPTH in (0, 256) else None
 
@@ -564,6 +567,8 @@ def run_ours(args):
                          "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
                          else "fallback 6.8 TB/s",
                          "kernel": kname, "bytes_per_attempt": BYTES_PER_ATTEMPT,
+                         "row_bytes_per_attempt": row_bytes, "row_frac": achieved / peak * row_bytes / BYTES_PER_ATTEMPT,
+                         "row_basis": "as frac, on the bytes of the spins as the kernel stores them",
                          "attempts_per_launch": attempts_per_launch, "avg_launch_ms": sweep_ms},
             "cpu_baseline": {"value": cpu_v, "unit": UNIT, "cores": cores, "kind": "oracle", "host": host_description(),
                              "sample": f"1 MCS of {cores} replicas (one per host thread) of the {L_SIDE}^3 lattice, "

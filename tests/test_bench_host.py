@@ -160,6 +160,14 @@ def test_headline_line_fields_and_arithmetic(fake_device, capsys, monkeypatch):
     assert [m.inst_base for m in made[1:]] == [0, bench.REPLICAS - 1]  # the plain leg's two replicas
 
 
+def test_headline_line_names_the_bytes_of_the_stored_rows(fake_device, capsys, monkeypatch):
+    monkeypatch.setattr(bench, "L_SIDE", 8)
+    bench.run_ours(args(mcs=2, side=8))
+    r = last_json(capsys)["roofline"]
+    assert r["kernel"] == "pass32_r32" and r["row_bytes_per_attempt"] == pytest.approx(25.5)
+    assert r["row_frac"] == pytest.approx(r["frac"] * 25.5 / 33.5)
+
+
 def test_quick_line(fake_device, capsys, monkeypatch):
     monkeypatch.setattr(bench, "L_SIDE", 6)
     bench.run_ours(args(mcs=1, steps=1, warmup=0, quick=True, side=6))
