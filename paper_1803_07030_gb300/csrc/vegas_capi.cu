@@ -2115,8 +2115,8 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                         set_cluster_shape(c, best_c.a, best_c.b, best_c.split, best_c.group, best_c.group * 16,
                                           best_c.sm != 0);
                     // The tiled form runs several times faster than the sweeps timed above wherever it
-                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 27.5, 55; the
-                    // 29k-site core/shell particle 4.9, 23; a 13k-site fcc sphere x 8 5.4, 24; 512 sites 2.1, 9),
+                    // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 25.8, 55; the
+                    // 29k-site core/shell particle 4.8, 23; a 13k-site fcc sphere x 8 5.3, 24; 512 sites 1.7, 9),
                     // so it is not timed: it takes the place of the one kept where it records what that
                     // one would.
                     if (!c->opt.resident_smem && tile_for(c, best_v)) {

@@ -16,8 +16,8 @@
 // per 32 threads. Large parts are bound by instruction issue (112 cycles per 32 attempts).
 //
 // us per MCS, before (grid barriers, neighbours in L2) and now: 64^3 with uniaxial anisotropy
-// 17.5 and 4.9, the 29k-site core/shell particle 23.0 and 4.9, a 13k-site fcc sphere x 8 replicas
-// 23.5 and 5.3, 128^3 54.6 and 27.5.
+// 17.5 and 4.9, the 29k-site core/shell particle 23.0 and 4.8, a 13k-site fcc sphere x 8 replicas
+// 23.5 and 5.3, 128^3 54.6 and 25.8.
 //
 // Why one mailbox word per site is enough: tag t + 1 marks the value after MCS t. Site i of part
 // N (class c) is read by part b because some site j of b (class c') links to i; then N reads j.
@@ -70,10 +70,11 @@ struct TilePrep {
 // keeps in shared memory beside the spins: 2 rows, site ids and remote words' indices, 1 the ids
 // and indices, 0 nothing (the rest is read through L1 from tables in the block's own order). FMT 1
 // halves the rows (samples of at most kTileCodes exchange values): for parts whose rows do not fit
-// otherwise, or are read from L2 (128^3, 100 MB of pairs: 46.8 us per MCS, 29.1 with words; 27.5 since
-// the warps add their sums, which leaves room for 512 threads in place of 384. There it is bound by
-// the warps that fit beside 12 bytes per spin: issue 45%. Slower: rows fetched a round ahead 30.9, two
-// sites in flight per thread 30.5; rows by link pair the same).
+// otherwise, or are read from L2 (128^3, 100 MB of pairs: 46.8 us per MCS, 29.1 with words; 27.5 once
+// the warps added their sums, which left room for 512 threads in place of 384; 25.8 without compensated
+// sums. There it is bound by the latency of an attempt with 16 sweeping warps per SM (issue 45%): kTileThreads
+// and their registers are the limit, a warp takes 36 bytes of shared memory beside 12 per spin. Slower, against
+// 27.5 to 28.8: rows fetched a round ahead 30.9, two sites in flight per thread 30.5; rows by link pair the same).
 template <int W, int POL, int PM, int MEM, int FMT>
 __global__ void __launch_bounds__(kTileThreads + kTileRecord) tile32_kernel(const TileArgs ta) {
     extern __shared__ __align__(16) unsigned char smem[];
