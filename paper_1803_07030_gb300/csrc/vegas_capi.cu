@@ -1848,6 +1848,12 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             CK(c, dalloc(c, &c->d_sched, sizeof(double) * sched.size()));
             c->sched_cap = sched.size();
         }
+        if (c->d_hist_t && hneed > c->hist_t_cap) {  // out of the way of what the run cannot do without
+            cudaFree(c->d_hist_t);
+            c->d_hist_t = nullptr;
+            c->device_bytes -= (int64_t)(c->hist_t_cap * sizeof(double) + c->hist_t_cap / 4 * sizeof(uint32_t));
+            c->hist_t_cap = 0;
+        }
         if (hneed > c->hist_cap) {
             if (c->d_hist) {
                 cudaFree(c->d_hist);
@@ -1888,11 +1894,6 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
             c->snap_cap = sneed;
         }
         if (NI > 1 && hneed > c->hist_t_cap) {  // the same records by instance, where there is room for them
-            if (c->d_hist_t) {
-                cudaFree(c->d_hist_t);
-                c->device_bytes -= (int64_t)(c->hist_t_cap * sizeof(double) + c->hist_t_cap / 4 * sizeof(uint32_t));
-            }
-            c->hist_t_cap = 0;
             CK(c, dalloc_spare(c, &c->d_hist_t, sizeof(double) * hneed + sizeof(uint32_t) * aneed));
             if (c->d_hist_t) c->hist_t_cap = hneed;
         }
@@ -2107,13 +2108,16 @@ extern "C" vegas_status vegas_run(vegas_ctx *c, const double *T, const double *B
                     // grouping of small instances
                     if (c->cluster_eligible && best_v != 3) set_cluster_shape(c, cs_rule, ct_rule, 0, 0, 0);
                     set_coop_shape(c, best_v == 2 ? best_c.a : 2);
-                    if (best_v == 1)
-                        set_resident_shape(c, best_c.a, best_c.group, best_c.group * 16, best_c.sm != 0);
-                    else
+                    auto shape = [&] {
+                        if (best_v == 1) return set_resident_shape(c, best_c.a, best_c.group, best_c.group * 16, best_c.sm != 0);
                         set_resident_shape(c, rt_rule);
-                    if (best_v == 3)
-                        set_cluster_shape(c, best_c.a, best_c.b, best_c.split, best_c.group, best_c.group * 16,
-                                          best_c.sm != 0);
+                        return best_v != 3 || set_cluster_shape(c, best_c.a, best_c.b, best_c.split, best_c.group,
+                                                                best_c.group * 16, best_c.sm != 0);
+                    };
+                    if (!shape()) {  // the batch kernel does not fit in that shape: the kernel that was timed does
+                        c->batch_ok = false;
+                        shape();
+                    }
                     // The tiled form runs several times faster than the sweeps timed above wherever it
                     // fits (us per MCS, and the best of the others: 64^3 4.9, 17.5; 128^3 25.8, 55; the
                     // 29k-site core/shell particle 4.8, 23; a 13k-site fcc sphere x 8 5.3, 24; 512 sites 1.7, 9),
