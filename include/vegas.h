@@ -70,7 +70,7 @@ typedef enum {
     VEGAS_ENOMEM = 2,   /* host or device allocation failed */
     VEGAS_ECUDA = 3,    /* a CUDA runtime call failed (no device, launch error, ...) */
     VEGAS_ETIMEOUT = 4, /* a bounded device wait ran out (grid barrier of the cooperative sweep,
-                           dependency wait of the wavefront sweep) */
+                           boundary spin of its tiled form, dependency wait of the wavefront sweep) */
     VEGAS_EDEVICE = 5,  /* a kernel flagged an error: NaN energy change, sampler cap */
     VEGAS_ESTATE = 6    /* context poisoned by an earlier ECUDA/EDEVICE/ETIMEOUT */
 } vegas_status;
@@ -130,7 +130,8 @@ typedef struct {
     void *cuda_stream;      /* cudaStream_t to run on, NULL = a stream of the library */
     int32_t variant;        /* -1 automatic: the first run times each eligible sweep and block
                                shape on a few MCS of the real chain and keeps the fastest
-                               (vegas_stats reports the choice); 0 one launch per colour
+                               (vegas_stats reports the choice; a kernel that adds the FP32 shares
+                               in the same order may run in its place); 0 one launch per colour
                                class, 1 resident: one persistent launch per step, a block per
                                instance (FP32), 2 cooperative: one launch per step, all blocks
                                sweep one sample class by class (FP32 or FP64, one sample, no
@@ -159,11 +160,12 @@ typedef struct {
                                flight per warp, 2 or 3; 1 = no staging (direct kernel);
                                0 = automatic. Default 0. */
     int64_t timeout_ns;     /* longest wait of a block at a grid barrier of the cooperative
-                               sweep, or of a warp for the dependencies of one block of the
+                               sweep or for a boundary spin of its tiled form, or of a warp for
+                               the dependencies of one block of the
                                wavefront sweep, before the run fails with VEGAS_ETIMEOUT;
                                0 = 2 s. */
     int32_t fault_inject;   /* testing only: 1 = in the cooperative sweep one block leaves
-                               before its first grid barrier, and in the wavefront sweep the
+                               before its first grid barrier or word, and in the wavefront sweep the
                                first block of class-0 sites is never reported finished, so the
                                blocks that wait for it time out; 2 = device buffers that only make
                                runs faster are not allocated, as when device memory is short.
